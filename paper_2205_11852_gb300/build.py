@@ -20,7 +20,7 @@ BUILD = PKG / "_build"
 LIB = BUILD / "libtpcf.so"
 
 SOURCES = ["api.cpp", "count.cpp", "plan.cpp", "mesh.cu", "paircount.cu", "pairdirect.cu", "estimator.cu",
-           "gram_split.cu", "noalloc.cu", "project.cu", "covcov.cu"]
+           "gram_split.cu", "gram_digits.cu", "noalloc.cu", "project.cu", "covcov.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

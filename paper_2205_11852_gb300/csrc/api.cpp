@@ -429,8 +429,14 @@ int tpcf_lc_cov(tpcf_ctx *ctx, const double *xi_a1, const double *xi_a2, const d
     if (M_a < 1) return fail(ctx, TPCF_ERR_ARG, "M_a must be >= 1");
     if (!(M >= (double)M_a)) return fail(ctx, TPCF_ERR_ARG, "M must be >= M_a (or +inf)");
     if (precision == TPCF_FP64) {
-        const int ns = fp64_splits(n_mock, nbin, 3);
         void *w;
+        if (cov_digits_suits(n_mock, nbin, 3, ctx->n_sm)) {
+            if ((rc = ensure(ctx, "lc_digits_work", cov_digits_work_bytes(n_mock, nbin, 3, ctx->n_sm), &w))) return rc;
+            CK(launch_cov_digits(xi_a1, xi_a2, xi_b, 3, n_mock, nbin, w, ctx->n_sm, M_a, M, C_lc, Ca, Cb, A, B,
+                                 ctx->status, s));
+            return TPCF_OK;
+        }
+        const int ns = fp64_splits(n_mock, nbin, 3);
         if ((rc = ensure(ctx, "lc_work", fp64_work_elems(n_mock, nbin, 3, ns) * 8, &w))) return rc;
         CK(launch_lc_fp64_split(xi_a1, xi_a2, xi_b, n_mock, nbin, (double *)w, ns, M_a, M, C_lc, Ca, Cb, A, B, s));
         return TPCF_OK;
@@ -457,8 +463,14 @@ int tpcf_sample_cov(tpcf_ctx *ctx, const double *xi, int n_mock, int nbin, int p
     if (n_mock < 2) return fail(ctx, TPCF_ERR_ARG, "n_mock must be >= 2");
     if (nbin < 1 || nbin > 65536) return fail(ctx, TPCF_ERR_ARG, "bad nbin");
     if (precision == TPCF_FP64) {
-        const int ns = fp64_splits(n_mock, nbin, 1);
         void *w;
+        if (cov_digits_suits(n_mock, nbin, 1, ctx->n_sm)) {
+            if ((rc = ensure(ctx, "lc_digits_work", cov_digits_work_bytes(n_mock, nbin, 1, ctx->n_sm), &w))) return rc;
+            CK(launch_cov_digits(xi, xi, xi, 1, n_mock, nbin, w, ctx->n_sm, 1, 2.0, C, nullptr, nullptr, nullptr,
+                                 nullptr, ctx->status, s));
+            return TPCF_OK;
+        }
+        const int ns = fp64_splits(n_mock, nbin, 1);
         if ((rc = ensure(ctx, "lc_work", fp64_work_elems(n_mock, nbin, 1, ns) * 8, &w))) return rc;
         CK(launch_cov_fp64(xi, n_mock, nbin, (double *)w, C, s, ns));
         return TPCF_OK;

@@ -202,6 +202,14 @@ cudaError_t launch_cov_fp64(const double *xi, int n_mock, int nbin, double *work
                             int n_split);
 cudaError_t launch_cov_split(const double *xi, int n_mock, int nbin, int precision, void *work, size_t work_bytes,
                              double *C, int *status, const GramOpts &opt, cudaStream_t s);
+// float64 covariances on the tensor cores from exact digit splits (gram_digits.cu): n_var = 3 the LC
+// covariance of (x0, x1, x2), n_var = 1 the sample covariance of x0 into C_lc; work holds
+// cov_digits_work_bytes(); cov_digits_suits: the sizes at which this is the faster float64 path
+bool cov_digits_suits(int n_mock, int nbin, int n_var, int n_sm);
+size_t cov_digits_work_bytes(int n_mock, int nbin, int n_var, int n_sm);
+cudaError_t launch_cov_digits(const double *x0, const double *x1, const double *x2, int n_var, int n_mock, int nbin,
+                              void *work, int n_sm, int M_a, double M, double *C_lc, double *Ca, double *Cb,
+                              double *A, double *B, int *status, cudaStream_t s);
 // column means mean[n_var][nbin] of the first n_var xi variants
 cudaError_t launch_means(const double *xi_a1, const double *xi_a2, const double *xi_b, int n_var, int n_mock,
                          int nbin, double *mean, cudaStream_t s);
