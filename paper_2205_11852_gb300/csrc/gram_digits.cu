@@ -58,10 +58,6 @@ constexpr int D_EPI_WARPS = 8;
 constexpr int D_THREADS = 32 * (D_EPI_WARPS + 2);
 constexpr int EXP_BAD = 1 << 20;               // "exponent" of a column that is not split
 
-struct CovOut {
-    double *p[5];   // C_lc, C^a, C^b, A, B (any but the first may be null)
-};
-
 static_assert(SEG_SLICES * DKS * 7 * 4096 < (1 << 24), "level sums must stay exact in FP32");
 
 // round(y 2^(55 - e)) for |y| < 2^e
@@ -317,9 +313,9 @@ __global__ void __launch_bounds__(D_THREADS, 1)
 
 // Adds the segments of T (integers) and combines: NV = 3 the LC covariance
 // (Eqs. R1R2, LCdef), NV = 1 the sample covariance into C_lc.  A block takes a
-// 16 x 16 tile of the lower triangle, one variant per layer of threads (all of
+// 8 x 8 tile of the lower triangle, one variant per layer of threads (all of
 // an element's loads in flight), and writes the tile and its mirror.
-constexpr int CT = 16;
+constexpr int CT = 8;
 template <int NV>
 __global__ void __launch_bounds__(CT *CT *NV)
     combine_digits_kernel(const longlong2 *__restrict__ T, int n_seg, int nbin, int n_mock,

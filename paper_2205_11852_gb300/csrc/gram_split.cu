@@ -9,13 +9,13 @@
 //   BF16X3: y = h + m + l (bf16 each), G ~ hh + hm + mh + hl + lh + mm  (6 products)
 // A CTA (one per SM) owns one 128 x 128 output tile of one variant and a
 // chunk of K-slices of 16 mocks: its operand tiles arrive by bulk copies
-// (cp.async.bulk, the TMA engine, completing on mbarriers) into two stages,
+// (cp.async.bulk, the TMA engine, completing on mbarriers) into four stages,
 // one thread issues each slice's tcgen05.mma chains into one of two FP32
 // accumulator sets in tensor memory, and eight warps read each finished set
-// back with tcgen05.ld and add it into a shared FP32 tile by compensated
-// (Kahan) summation while the next slice multiplies; the tile becomes the
-// chunk's partial Gram, which a reduction kernel sums over the chunks in
-// float64, in chunk order.  The leading product (hi.hi) and the much smaller
+// back with tcgen05.ld and add it into sums in registers by compensated
+// (Kahan) summation while the next slice multiplies; the sums become the
+// chunk's partial Gram, and the combining kernel adds the chunks in float64,
+// in chunk order.  The leading product (hi.hi) and the much smaller
 // correction products go to two separate accumulators, so the FP32 rounding of
 // an accumulator spans one slice's exact products and the corrections do not
 // round against the leading sum.
@@ -29,6 +29,7 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "colstats.cuh"
 #include "tc_ptx.cuh"
 #include "tpcf_internal.h"
 
@@ -39,10 +40,9 @@ constexpr int TM = 128;          // rows (bins) per tile, M = N of the MMA
 constexpr int KS = 16;           // mocks per K-slice
 constexpr int TMEM_COLS = 4 * TM; // two accumulator sets of (leading product, corrections)
 constexpr int GRAM_EPI_WARPS = 8;  // the epilogue: warp w reads TMEM lanes 32 (w mod 4).. and columns half w / 4
-constexpr int GRAM_THREADS = 32 * (GRAM_EPI_WARPS + 1);   // + one warp for the loads and MMAs
+constexpr int GRAM_THREADS = 32 * (GRAM_EPI_WARPS + 2);   // + one warp for the MMAs and one for the loads
 static_assert(GRAM_EPI_WARPS == 8 && TM == 128, "two warpgroups split a 128-column tile (drain and store)");
-constexpr int NSTAGE = 2;                    // K-slices in flight per CTA
-constexpr int TPAD = TM + 1;                 // row stride (floats) of the shared tile
+constexpr int NSTAGE = 4;                    // K-slices in flight per CTA
 
 template <int PREC>
 struct Split;
@@ -91,43 +91,124 @@ __device__ __forceinline__ uint32_t tf32_rna(float x)
     return y;
 }
 
-// centred residuals, split into pieces, written as operand tiles
-// tiles[v][piece][rb][ks]
-template <int PREC>
-__global__ void split_kernel(const double *__restrict__ x0, const double *__restrict__ x1,
-                             const double *__restrict__ x2, const double *__restrict__ mean, int n_mock, int nbin,
-                             int n_rb, int n_ks, unsigned char *__restrict__ tiles)
+// The splits of a residual, on the integer pipes where its exponent allows
+// (|d| in [2^-74, 2^126]; the float64 pipe, one to two operations per clock
+// and SM with its conversions, bounded the split kernel: 30 us at 3500 x 200).
+// The remainders stay exact integers in units of d's last place, so the pieces
+// equal those of float64 subtractions and conversions bit for bit.
+struct Int64Parts {
+    bool plain;       // the integer path applies
+    int sign;         // 0x80000000 for a negative d
+    uint32_t ex;      // biased float64 exponent
+    long long m;      // 53-bit magnitude
+    float ulp;        // weight of m's last bit
+
+    __device__ __forceinline__ explicit Int64Parts(double d)
+    {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(d);
+        ex = (uint32_t)(b >> 52) & 0x7ffu;
+        plain = ex - 949u <= 200u;
+        sign = (int)((uint32_t)(b >> 32) & 0x80000000u);
+        m = (long long)((b & 0xfffffffffffffull) | (1ull << 52));
+        ulp = __uint_as_float((ex - 948u) << 23);
+    }
+};
+
+// hi = rna_tf32((float)d), lo = rna_tf32((float)(d - hi))
+__device__ __forceinline__ void split_tf32(double d, uint32_t &hi, uint32_t &lo)
 {
-    const int v = blockIdx.z;
-    const double *x = v == 0 ? x0 : (v == 1 ? x1 : x2);
-    const int rb = blockIdx.y, ks = blockIdx.x;
+    const Int64Parts q(d);
+    if (!q.plain) {
+        hi = tf32_rna((float)d);
+        lo = tf32_rna((float)(d - (double)__uint_as_float(hi)));
+        return;
+    }
+    // the float nearest to |d| (ties to even)
+    const unsigned long long u = (unsigned long long)q.m + 0x0fffffffull + (((unsigned long long)q.m >> 29) & 1ull);
+    const uint32_t h = tf32_rna(__uint_as_float((uint32_t)(u >> 29) + ((q.ex - 897u) << 23)));
+    const long long r = q.m - ((long long)((h & 0x7fffffu) | 0x800000u) << ((h >> 23) - q.ex + 925u));
+    hi = h | (uint32_t)q.sign;
+    lo = tf32_rna(__ll2float_rn(r) * q.ulp) ^ (uint32_t)q.sign;
+}
+
+// three bf16 pieces, each the nearest to the remainder of the ones before
+__device__ __forceinline__ void split_bf16(double d, uint16_t (&p)[3])
+{
+    const Int64Parts q(d);
+    if (!q.plain) {
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            const __nv_bfloat16 t = __double2bfloat16(d);
+            d -= (double)__bfloat162float(t);
+            p[k] = __bfloat16_as_ushort(t);
+        }
+        return;
+    }
+    long long r = q.m;
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        // truncated to a float with a sticky last bit, which bf16 then rounds correctly
+        const float f = __ll2float_rz(r);
+        const uint32_t sticky = __float2ll_rz(f) != r ? 1u : 0u;
+        const float t = __bfloat162float(__float2bfloat16_rn(__uint_as_float(__float_as_uint(f) | sticky)));
+        r -= __float2ll_rz(t);   // exact: t has no bits below r's last place
+        p[k] = (uint16_t)((__float_as_uint(t * q.ulp) ^ (uint32_t)q.sign) >> 16);
+    }
+}
+
+// centred residuals, split into pieces, written as operand tiles
+// tiles[v][piece][rb][ks].  A block takes 32 columns (one per lane) and one of
+// COL_CHUNKS row ranges of one variant, closes the column statistics of all
+// row ranges (colstats.cuh) and writes whole 16-byte core-matrix rows: `per`
+// consecutive mocks of one bin.  Rows past nbin are left unwritten (an output
+// element depends on its own two operand rows only), mocks past n_mock are
+// zeros.
+template <int PREC>
+__global__ void __launch_bounds__(32 * COL_WARPS)
+    split_kernel(const double *__restrict__ x0, const double *__restrict__ x1, const double *__restrict__ x2,
+                 const ColPartial *__restrict__ part, int n_mock, int nbin, int n_rb, int n_ks,
+                 unsigned char *__restrict__ tiles)
+{
     constexpr int TB = tile_bytes<PREC>();
     constexpr int NP = Split<PREC>::PIECES;
-    for (int e = threadIdx.x; e < TM * KS; e += blockDim.x) {
-        const int r = e % TM, k = e / TM;
-        const int i = rb * TM + r, m = ks * KS + k;
-        const double y = (i < nbin && m < n_mock) ? x[(size_t)m * nbin + i] - mean[(size_t)v * nbin + i] : 0.0;
-        const uint32_t off = tile_offset<PREC>(r, k);
+    constexpr int per = 16 / Split<PREC>::ELEM;
+    const int v = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double *x = v == 0 ? x0 : (v == 1 ? x1 : x2);
+    const int b = blockIdx.x * 32 + lane;
+    double mu, mn, mx;
+    column_stats(part, v, n_mock, nbin, b, mu, mn, mx);
+    if (b >= nbin) return;
+    const int rb = b / TM, r = b % TM;
+    const int n_g = n_ks * (KS / per), share = (n_g + (int)gridDim.y - 1) / (int)gridDim.y;
+    const int g1 = min(n_g, ((int)blockIdx.y + 1) * share);
+#pragma unroll 2
+    for (int g = (int)blockIdx.y * share + warp; g < g1; g += COL_WARPS) {
+        const int m0 = g * per, ks = m0 / KS;
+        double y[per];
+#pragma unroll
+        for (int k = 0; k < per; k++) y[k] = m0 + k < n_mock ? x[(size_t)(m0 + k) * nbin + b] : mu;
+        uint32_t w[NP][4];
         if (PREC == TPCF_TF32X3) {
-            const uint32_t hi = tf32_rna((float)y);
-            const uint32_t lo = tf32_rna((float)(y - (double)__uint_as_float(hi)));
-            unsigned char *t0 = tiles + ((((size_t)v * NP + 0) * n_rb + rb) * n_ks + ks) * TB;
-            unsigned char *t1 = tiles + ((((size_t)v * NP + 1) * n_rb + rb) * n_ks + ks) * TB;
-            *(uint32_t *)(t0 + off) = hi;
-            *(uint32_t *)(t1 + off) = lo;
+#pragma unroll
+            for (int k = 0; k < per; k++) {
+                const double d = m0 + k < n_mock ? y[k] - mu : 0.0;
+                split_tf32(d, w[0][k], w[1][k]);
+            }
         } else {
-            const __nv_bfloat16 h = __double2bfloat16(y);
-            const double r1 = y - (double)__bfloat162float(h);
-            const __nv_bfloat16 mm = __double2bfloat16(r1);
-            const double r2 = r1 - (double)__bfloat162float(mm);
-            const __nv_bfloat16 l = __double2bfloat16(r2);
-            unsigned char *t0 = tiles + ((((size_t)v * NP + 0) * n_rb + rb) * n_ks + ks) * TB;
-            unsigned char *t1 = tiles + ((((size_t)v * NP + 1) * n_rb + rb) * n_ks + ks) * TB;
-            unsigned char *t2 = tiles + ((((size_t)v * NP + 2) * n_rb + rb) * n_ks + ks) * TB;
-            *(__nv_bfloat16 *)(t0 + off) = h;
-            *(__nv_bfloat16 *)(t1 + off) = mm;
-            *(__nv_bfloat16 *)(t2 + off) = l;
+            uint16_t h[per][3];
+#pragma unroll
+            for (int k = 0; k < per; k++) split_bf16(m0 + k < n_mock ? y[k] - mu : 0.0, h[k]);
+#pragma unroll
+            for (int p = 0; p < NP; p++)
+#pragma unroll
+                for (int k = 0; k < 4; k++)
+                    w[p][k] = (uint32_t)h[(2 * k) % per][p] | (uint32_t)h[(2 * k + 1) % per][p] << 16;
         }
+        const uint32_t off = tile_offset<PREC>(r, m0 % KS);
+#pragma unroll
+        for (int p = 0; p < NP; p++)
+            *(uint4 *)(tiles + ((((size_t)v * NP + p) * n_rb + rb) * n_ks + ks) * TB + off) =
+                make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
     }
 }
 
@@ -163,23 +244,46 @@ __host__ __device__ constexpr uint32_t instr_desc()
 template <int PREC>
 __host__ __device__ constexpr int stage_bytes() { return 2 * Split<PREC>::PIECES * tile_bytes<PREC>(); }
 
-// shared memory: NSTAGE stages | FP32 tile sums and compensations [2][TM][TPAD] | full[NSTAGE], empty[NSTAGE],
-// accf[2], accfree[2], done barriers | TMEM slot | flags
+// shared memory: NSTAGE stages | full[NSTAGE], empty[NSTAGE], accf[2], accfree[2], done barriers | TMEM slot | flag
 template <int PREC>
-constexpr int gram_smem_bytes() { return NSTAGE * stage_bytes<PREC>() + 8 * TM * TPAD + 8 * (2 * NSTAGE + 5) + 16; }
+constexpr int gram_smem_bytes() { return NSTAGE * stage_bytes<PREC>() + 8 * (2 * NSTAGE + 5) + 16; }
+
+// 16 columns of both accumulators of a set, complete on return
+__device__ __forceinline__ void tmem_ld16x2(uint32_t t, uint32_t (&lo)[16], uint32_t (&hi)[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15}, [%32];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, "
+        "%29, %30, %31}, [%33];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(lo[0]), "=r"(lo[1]), "=r"(lo[2]), "=r"(lo[3]), "=r"(lo[4]), "=r"(lo[5]), "=r"(lo[6]), "=r"(lo[7]),
+          "=r"(lo[8]), "=r"(lo[9]), "=r"(lo[10]), "=r"(lo[11]), "=r"(lo[12]), "=r"(lo[13]), "=r"(lo[14]),
+          "=r"(lo[15]), "=r"(hi[0]), "=r"(hi[1]), "=r"(hi[2]), "=r"(hi[3]), "=r"(hi[4]), "=r"(hi[5]), "=r"(hi[6]),
+          "=r"(hi[7]), "=r"(hi[8]), "=r"(hi[9]), "=r"(hi[10]), "=r"(hi[11]), "=r"(hi[12]), "=r"(hi[13]),
+          "=r"(hi[14]), "=r"(hi[15])
+        : "r"(t), "r"(t + TM)
+        : "memory");
+}
 
 // One CTA (one per SM): output tile (bi, bj) of variant v over the K-slices
-// [k0, k0 + n) of chunk kc.  Warp 4 keeps NSTAGE slices of operand tiles in
-// flight (bulk copies completing on full[stage]) and issues each slice's MMA
-// chain into accumulator set i % 2 of tensor memory (columns 256 (i % 2) +
+// [k0, k0 + n) of chunk kc.  Warp 9 keeps NSTAGE slices of operand tiles in
+// flight (bulk copies completing on full[stage]); warp 8 issues each slice's
+// MMA chain into accumulator set i % 2 of tensor memory (columns 256 (i % 2) +
 // [0, 128): leading product, + [128, 256): corrections), once the epilogue has
-// drained that set's previous slice (accfree).  Warps 0-3 (TMEM lanes = tile
-// rows) read each finished set (accf) and add its two accumulators into a
-// shared [column][row] tile by compensated (Kahan) FP32 summation (the FP64
-// pipe is too slow for this on the SMs), so the tile holds the chunk's sum to
-// about one FP32 rounding while the tensor cores work on slice i + 1.  At the end the
-// tile is written to P[kc][v] (both triangles) with stores of 32 consecutive
-// doubles per warp.
+// drained that set's previous slice (accfree).  Warps 0-7 (TMEM lanes = tile
+// rows, two halves of the columns) read each finished set (accf) and add its
+// two accumulators into 64 register sums per thread by compensated (Kahan)
+// FP32 summation (the FP64 pipe is too slow for this on the SMs), so the sums
+// hold the chunk to about one FP32 rounding while the tensor cores work on
+// slice i + 1.  At the end D(row i, column j) goes to P[kc][v][j][i], 32
+// consecutive doubles per warp.
+//
+// The drain bounds it: per slice 2 x 16384 accumulator values against 8
+// additions each.  With the sums in shared memory (16 bytes of traffic per
+// element and slice) and the loads issued by the MMA thread only after the
+// slice's products had finished, the kernel took 46 us (3500 x 200, TF32x3),
+// now 31 us; the whole covariance 129 -> 69 us.
 //
 // Every wait is bounded.  The epilogue's waits for the products give up after
 // done_limit polls (a context option); skip_mma (tests only) makes CTA
@@ -195,15 +299,13 @@ __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const unsigned
     constexpr int NP = Split<PREC>::PIECES;
     constexpr int SB = stage_bytes<PREC>();
     extern __shared__ __align__(128) unsigned char smem[];
-    float *tsum = (float *)(smem + NSTAGE * SB);              // [TM columns][TPAD]
-    float *tcmp = tsum + TM * TPAD;                           // Kahan compensations, same layout
-    uint64_t *full = (uint64_t *)(tcmp + TM * TPAD);
+    uint64_t *full = (uint64_t *)(smem + NSTAGE * SB);
     uint64_t *empty = full + NSTAGE;
     uint64_t *accf = empty + NSTAGE;
     uint64_t *accfree = accf + 2;
     uint64_t *done = accfree + 2;
     uint32_t *slot = (uint32_t *)(done + 1);
-    int *flag = (int *)(slot + 1);   // [0]: a done commit was issued or skipped on purpose, [1]: all slices multiplied
+    int *all_in = (int *)(slot + 1);   // every slice was multiplied
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // blockIdx.x enumerates the upper-triangle tile pairs (bi <= bj) row by row
@@ -229,37 +331,48 @@ __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const unsigned
         }
         mbar_init(done, 1);
         mbar_fence_init();
-        flag[0] = 0;
-        flag[1] = 0;
+        *all_in = 0;
     }
-    for (int e = tid; e < 2 * TM * TPAD; e += blockDim.x) tsum[e] = 0.0f;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *slot;
+    bool fine = true;
+    float sum[TM / 2], cmp[TM / 2];   // the epilogue's column half of this thread's row
 
-    if (warp == GRAM_EPI_WARPS) {
+    if (warp == GRAM_EPI_WARPS + 1) {
         if (lane == 0) {
-            auto issue = [&](int i) {   // the operand tiles of slice k0 + i into stage i % NSTAGE
-                unsigned char *sa = smem + (i % NSTAGE) * SB, *sb = sa + NP * TB;
-                mbar_expect_tx(&full[i % NSTAGE], (uint32_t)SB);
+            const int n_load = skip ? min(NSTAGE, n) : n;
+            int issued = 0;
+            bool ok = true;
+            for (; issued < n_load; issued++) {   // the operand tiles of slice k0 + issued
+                const int st = issued % NSTAGE;
+                if (issued >= NSTAGE) {
+                    ok = mbar_wait(&empty[st], (uint32_t)(issued / NSTAGE - 1) & 1u, SPIN_LIMIT);
+                    if (!ok) break;
+                }
+                unsigned char *sa = smem + st * SB, *sb = sa + NP * TB;
+                mbar_expect_tx(&full[st], (uint32_t)SB);
                 for (int p = 0; p < NP; p++) {
                     const size_t base = ((size_t)v * NP + p) * n_rb;
-                    bulk_g2s(sa + p * TB, tiles + ((base + bi) * n_ks + k0 + i) * TB, TB, &full[i % NSTAGE]);
-                    bulk_g2s(sb + p * TB, tiles + ((base + bj) * n_ks + k0 + i) * TB, TB, &full[i % NSTAGE]);
+                    bulk_g2s(sa + p * TB, tiles + ((base + bi) * n_ks + k0 + issued) * TB, TB, &full[st]);
+                    bulk_g2s(sb + p * TB, tiles + ((base + bj) * n_ks + k0 + issued) * TB, TB, &full[st]);
                 }
-            };
-            int issued = 0, waited = 0, mma_slices = 0;
+            }
+            if (!ok) {   // the copies in flight land before the block may leave (bounded)
+                atomicOr(status, STATUS_TIMEOUT);
+                for (int i = max(0, issued - NSTAGE); i < issued; i++)
+                    mbar_wait(&full[i % NSTAGE], (uint32_t)(i / NSTAGE) & 1u, SPIN_LIMIT);
+            }
+        }
+    } else if (warp == GRAM_EPI_WARPS) {
+        if (lane == 0) {
             bool ok = true;
-            for (; issued < min(NSTAGE, n); issued++) issue(issued);
             for (int i = 0; i < n; i++) {
+                if (skip && i == NSTAGE) break;
                 ok = mbar_wait(&full[i % NSTAGE], (uint32_t)(i / NSTAGE) & 1u, SPIN_LIMIT);
                 if (!ok) break;
-                waited = i + 1;
-                if (skip) {
-                    if (waited == issued) break;   // every copy in flight has landed
-                    continue;
-                }
+                if (skip) continue;
                 // accumulator set i % 2 is free once the epilogue has drained slice i - 2
                 if (i >= 2) {
                     ok = mbar_wait(&accfree[i % 2], (uint32_t)((i - 2) / 2) & 1u, SPIN_LIMIT);
@@ -288,27 +401,17 @@ __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const unsigned
                 }
                 mma_commit(&empty[i % NSTAGE]);
                 mma_commit(&accf[i % 2]);
-                mma_slices = i + 1;
-                if (issued < n) {   // refill this stage once its products have read it
-                    ok = mbar_wait(&empty[i % NSTAGE], (uint32_t)(i / NSTAGE) & 1u, SPIN_LIMIT);
-                    if (!ok) break;
-                    issue(issued++);
-                }
             }
-            if (mma_slices > 0) mma_commit(done);
-            // copies still in flight after a wait gave up get one more bounded wait each
-            for (int i = waited; i < issued; i++)
-                if (!mbar_wait(&full[i % NSTAGE], (uint32_t)(i / NSTAGE) & 1u, SPIN_LIMIT)) break;
-            flag[0] = (mma_slices > 0 || skip) ? 1 : 0;
-            flag[1] = (ok && mma_slices == n) ? 1 : 0;
+            *all_in = (ok && !skip) ? 1 : 0;
+            if (!skip) mma_commit(done);   // also when a wait gave up: what was issued completes before TMEM is freed
             if (!ok) atomicOr(status, STATUS_TIMEOUT);
         }
     } else {
         // epilogue: row = this thread's TMEM lane; the two warpgroups take the
         // columns [0, TM / 2) and [TM / 2, TM) of both accumulators
-        const int wr = warp & 3, c_lo = (warp >> 2) * (TM / 2);
-        const int r = wr * 32 + lane;
-        bool fine = true;
+        const uint32_t lane0 = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * (TM / 2));
+#pragma unroll
+        for (int c = 0; c < TM / 2; c++) sum[c] = cmp[c] = 0.0f;
         for (int i = 0; i < n && fine; i++) {
             fine = mbar_wait(&accf[i % 2], (uint32_t)(i / 2) & 1u, done_limit);
             if (!fine) {
@@ -316,26 +419,22 @@ __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const unsigned
                 if (!fine) break;
             }
             tc_fence_after();
-            const uint32_t set = tmem + ((uint32_t)(wr * 32) << 16) + (uint32_t)((i % 2) * 2 * TM);
-#pragma unroll 1
-            for (int c0 = c_lo; c0 < c_lo + TM / 2; c0 += 32) {
-                uint32_t lo[32], hi[32];
-                tmem_ld32(set + (uint32_t)c0, lo);
-                tmem_ld32(set + (uint32_t)(TM + c0), hi);
 #pragma unroll
-                for (int j = 0; j < 32; j++) {
-                    const int e = (c0 + j) * TPAD + r;
-                    float sum = tsum[e], cmp = tcmp[e];
+            for (int c0 = 0; c0 < TM / 2; c0 += 16) {
+                uint32_t lo[16], hi[16];
+                tmem_ld16x2(lane0 + (uint32_t)((i % 2) * 2 * TM + c0), lo, hi);
+#pragma unroll
+                for (int j = 0; j < 16; j++) {
                     // two compensated additions (the leading product, then the corrections)
-                    float y = __fsub_rn(__uint_as_float(lo[j]), cmp);
-                    float t = __fadd_rn(sum, y);
-                    cmp = __fsub_rn(__fsub_rn(t, sum), y);
-                    sum = t;
-                    y = __fsub_rn(__uint_as_float(hi[j]), cmp);
-                    t = __fadd_rn(sum, y);
-                    cmp = __fsub_rn(__fsub_rn(t, sum), y);
-                    tsum[e] = t;
-                    tcmp[e] = cmp;
+                    float sm = sum[c0 + j], cp = cmp[c0 + j];
+                    float y = __fsub_rn(__uint_as_float(lo[j]), cp);
+                    float t = __fadd_rn(sm, y);
+                    cp = __fsub_rn(__fsub_rn(t, sm), y);
+                    sm = t;
+                    y = __fsub_rn(__uint_as_float(hi[j]), cp);
+                    t = __fadd_rn(sm, y);
+                    cmp[c0 + j] = __fsub_rn(__fsub_rn(t, sm), y);
+                    sum[c0 + j] = t;
                 }
             }
             tc_fence_before();
@@ -346,34 +445,20 @@ __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const unsigned
     }
     __syncthreads();
     // every product has completed before tensor memory is released (bounded)
-    bool good = flag[1] != 0;
-    if (flag[0]) {
+    bool good = *all_in != 0;
+    if (!skip) {
         bool fin = mbar_wait(done, 0, done_limit);
         if (!fin) fin = mbar_wait(done, 0, done_limit);
         good = good && fin;
     }
     if (!good && tid == 0) atomicOr(status, STATUS_TIMEOUT);
-    if (good && warp < GRAM_EPI_WARPS) {
+    if (good && fine && warp < GRAM_EPI_WARPS) {
         double *g = P + ((size_t)kc * gridDim.y + v) * nbin * nbin;
-        // the epilogue warps' 256 threads: t in [0, TM) and a half h of the other index
-        const int t = (warp * 32 + lane) & (TM - 1), h0 = ((warp * 32 + lane) / TM) * (TM / 2);
-        // the block itself: thread t takes column t (consecutive threads, consecutive doubles)
-        const int col = bj * TM + t;
-        if (col < nbin) {
-            for (int rr = h0; rr < h0 + TM / 2; rr++) {
-                const int row = bi * TM + rr;
-                if (row >= nbin) break;
-                g[(size_t)row * nbin + col] = (double)tsum[t * TPAD + rr] - (double)tcmp[t * TPAD + rr];
-            }
-        }
-        // the transposed block of an off-diagonal pair: thread t takes row t
-        const int row = bi * TM + t;
-        if (bi != bj && row < nbin) {
-            for (int c = h0; c < h0 + TM / 2; c++) {
-                const int cc = bj * TM + c;
-                if (cc >= nbin) break;
-                g[(size_t)cc * nbin + row] = (double)tsum[c * TPAD + t] - (double)tcmp[c * TPAD + t];
-            }
+        const int row = bi * TM + (warp & 3) * 32 + lane, col0 = bj * TM + (warp >> 2) * (TM / 2);
+        if (row < nbin) {
+#pragma unroll
+            for (int c = 0; c < TM / 2; c++)
+                if (col0 + c < nbin) g[(size_t)(col0 + c) * nbin + row] = (double)sum[c] - (double)cmp[c];
         }
     }
     tc_fence_before();
@@ -381,13 +466,62 @@ __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const unsigned
     if (warp == 0) tmem_dealloc(tmem, TMEM_COLS);
 }
 
-// G[v][i][j] = sum over the chunks kc of P[kc][v][i][j], in chunk order (deterministic)
-__global__ void reduce_partials_kernel(const double *__restrict__ P, int n_kc, size_t per, double *__restrict__ G)
+// Adds the chunks' partials in chunk order (float64, deterministic) and
+// combines: NV = 3 the LC covariance (Eqs. R1R2, LCdef), NV = 1 the sample
+// covariance into out.p[0].  P[kc][v][j][i] = D(i, j) for the 128-tiles
+// (i, j) with i's tile <= j's tile; an element below the diagonal tiles is the
+// mirror of the one above.  A block takes an 8 x 8 tile (r in [8 tr, +8), c in
+// [8 tc, +8), tc >= tr; with 16 x 16 the 91 blocks of 200 bins left SMs idle
+// under the float64 additions: 20 us), one variant per layer of threads, and writes it
+// and its mirror.
+constexpr int CT = 8;
+template <int NV>
+__global__ void __launch_bounds__(CT *CT *NV) combine_partials_kernel(const double *__restrict__ P, int n_kc, int nbin,
+                                                                     int n_mock, int M_a, double M, CovOut out)
 {
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < per; e += (size_t)gridDim.x * blockDim.x) {
+    __shared__ double sc[NV][2][CT][CT + 1];
+    int tc = (int)((sqrtf(8.0f * (float)blockIdx.x + 1.0f) - 1.0f) * 0.5f);
+    while ((long long)tc * (tc + 1) / 2 > (long long)blockIdx.x) tc--;
+    while ((long long)(tc + 1) * (tc + 2) / 2 <= (long long)blockIdx.x) tc++;
+    const int tr = (int)((long long)blockIdx.x - (long long)tc * (tc + 1) / 2);   // tr <= tc
+    const int v = threadIdx.x / (CT * CT), tx = threadIdx.x % CT, ty = threadIdx.x / CT % CT;
+    const size_t nn = (size_t)nbin * nbin;
+    const double inv = 1.0 / (double)(n_mock - 1);
+    const bool same = tr / (TM / CT) == tc / (TM / CT);   // inside a diagonal 128-tile: both triangles are stored
+#pragma unroll
+    for (int h = 0; h < 2; h++) {   // h = 0: D(row r, column c); 1: D(row c, column r), inside a diagonal tile only
+        if (h && (!same || tr == tc)) break;
+        const int i = (h ? tc : tr) * CT + tx, j = (h ? tr : tc) * CT + ty;
         double acc = 0.0;
-        for (int k = 0; k < n_kc; k++) acc += P[(size_t)k * per + e];
-        G[e] = acc;
+        if (i < nbin && j < nbin) {
+            const double *p = P + (size_t)v * nn + (size_t)j * nbin + i;
+#pragma unroll 8
+            for (int k = 0; k < n_kc; k++) acc += p[(size_t)k * NV * nn];
+        }
+        sc[v][h][ty][tx] = acc * inv;   // [column][row]
+    }
+    __syncthreads();
+    // out(row, col): tile (tr, tc) from h = 0 transposed; tile (tc, tr) from h = 1 transposed, or the mirror of h = 0
+    for (int w = v; w < 2; w += NV) {
+        if (w && tr == tc) break;
+        const int row = (w ? tc : tr) * CT + ty, col = (w ? tr : tc) * CT + tx;
+        if (row >= nbin || col >= nbin) continue;
+        double c[3];
+#pragma unroll
+        for (int q = 0; q < NV; q++) c[q] = w == 0 ? sc[q][0][tx][ty] : (same ? sc[q][1][tx][ty] : sc[q][0][ty][tx]);
+        const size_t t = (size_t)row * nbin + col;
+        if (NV == 1) {
+            out.p[0][t] = c[0];
+            continue;
+        }
+        const double ca = 0.5 * c[0] + 0.5 * c[NV / 3], cb = c[NV - 1];
+        const double a = 2.0 * cb - ca;
+        const double bb = 2.0 * (double)M_a * (ca - cb);
+        out.p[0][t] = a + bb / M;
+        if (out.p[1]) out.p[1][t] = ca;
+        if (out.p[2]) out.p[2][t] = cb;
+        if (out.p[3]) out.p[3][t] = a;
+        if (out.p[4]) out.p[4][t] = bb;
     }
 }
 
@@ -425,8 +559,8 @@ size_t work_bytes_of(int n_mock, int nbin, int n_var, int n_sm)
 {
     const Chunking c = chunking(n_mock, nbin, n_var, n_sm);
     const size_t g = (size_t)n_var * nbin * nbin * 8;
-    return al256(tiles_bytes<PREC>(n_mock, nbin, n_var)) + al256(g) + al256((size_t)c.n_kc * g) +
-           al256((size_t)n_var * nbin * 8);
+    return al256(tiles_bytes<PREC>(n_mock, nbin, n_var)) + al256((size_t)c.n_kc * g) +
+           al256((size_t)n_var * COL_CHUNKS * nbin * sizeof(ColPartial));
 }
 
 // n_var = 3: the LC covariance of (x0, x1, x2); n_var = 1: the sample covariance of x0 into C_lc
@@ -443,16 +577,17 @@ cudaError_t run(const double *x0, const double *x1, const double *x2, int n_var,
     unsigned char *tiles = w;
     const size_t g = (size_t)n_var * nbin * nbin;
     size_t o = al256(tiles_bytes<PREC>(n_mock, nbin, n_var));
-    double *G = (double *)(w + o);
-    o += al256(g * 8);
     double *P = (double *)(w + o);
     o += al256((size_t)ch.n_kc * g * 8);
-    double *mean = (double *)(w + o);
-    o += al256((size_t)n_var * nbin * 8);
+    ColPartial *part = (ColPartial *)(w + o);
+    o += al256((size_t)n_var * COL_CHUNKS * nbin * sizeof(ColPartial));
     if (o > work_bytes) return cudaErrorInvalidValue;
-    cudaError_t e = launch_means(x0, x1, x2, n_var, n_mock, nbin, mean, s);
+    cudaError_t e = launch_column_partials(x0, x1, x2, n_var, n_mock, nbin, part, s);
     if (e != cudaSuccess) return e;
-    split_kernel<PREC><<<dim3(n_ks, n_rb, n_var), 256, 0, s>>>(x0, x1, x2, mean, n_mock, nbin, n_rb, n_ks, tiles);
+    split_kernel<PREC><<<dim3((nbin + 31) / 32, COL_CHUNKS, n_var), 32 * COL_WARPS, 0, s>>>(x0, x1, x2, part, n_mock,
+                                                                                           nbin, n_rb, n_ks, tiles);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     const int np = n_rb * (n_rb + 1) / 2;   // upper-triangle tile pairs
     const int smem = gram_smem_bytes<PREC>();
     e = cudaFuncSetAttribute(gram_tc_kernel<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -462,12 +597,14 @@ cudaError_t run(const double *x0, const double *x1, const double *x2, int n_var,
         opt.test_skip_mma);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int rb = (int)std::min<size_t>((g + 255) / 256, 4096);
-    reduce_partials_kernel<<<rb, 256, 0, s>>>(P, ch.n_kc, g, G);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (n_var == 1) return launch_scale(G, nbin, n_mock, C_lc, s);
-    return launch_combine(G, nbin, n_mock, M_a, M, C_lc, Ca, Cb, A, B, s);
+    const long long nt = (nbin + CT - 1) / CT;
+    const unsigned nb = (unsigned)(nt * (nt + 1) / 2);
+    const CovOut out{{C_lc, Ca, Cb, A, B}};
+    if (n_var == 3)
+        combine_partials_kernel<3><<<nb, CT * CT * 3, 0, s>>>(P, ch.n_kc, nbin, n_mock, M_a, M, out);
+    else
+        combine_partials_kernel<1><<<nb, CT * CT, 0, s>>>(P, ch.n_kc, nbin, n_mock, M_a, M, out);
+    return cudaGetLastError();
 }
 
 }  // namespace

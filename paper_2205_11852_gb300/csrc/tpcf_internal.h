@@ -202,6 +202,10 @@ cudaError_t launch_cov_fp64(const double *xi, int n_mock, int nbin, double *work
                             int n_split);
 cudaError_t launch_cov_split(const double *xi, int n_mock, int nbin, int precision, void *work, size_t work_bytes,
                              double *C, int *status, const GramOpts &opt, cudaStream_t s);
+// outputs of a covariance: C_lc, C^a, C^b, A, B (any but the first may be null)
+struct CovOut {
+    double *p[5];
+};
 // float64 covariances on the tensor cores from exact digit splits (gram_digits.cu): n_var = 3 the LC
 // covariance of (x0, x1, x2), n_var = 1 the sample covariance of x0 into C_lc; work holds
 // cov_digits_work_bytes(); cov_digits_suits: the sizes at which this is the faster float64 path
@@ -210,15 +214,6 @@ size_t cov_digits_work_bytes(int n_mock, int nbin, int n_var, int n_sm);
 cudaError_t launch_cov_digits(const double *x0, const double *x1, const double *x2, int n_var, int n_mock, int nbin,
                               void *work, int n_sm, int M_a, double M, double *C_lc, double *Ca, double *Cb,
                               double *A, double *B, int *status, cudaStream_t s);
-// column means mean[n_var][nbin] of the first n_var xi variants
-cudaError_t launch_means(const double *xi_a1, const double *xi_a2, const double *xi_b, int n_var, int n_mock,
-                         int nbin, double *mean, cudaStream_t s);
-// LC combination from the three Gram blocks G[3][nbin][nbin] (float64)
-cudaError_t launch_combine(const double *G, int nbin, int n_mock, int M_a, double M, double *C_lc, double *Ca,
-                           double *Cb, double *A, double *B, cudaStream_t s);
-// C = G / (n_mock - 1) for one Gram block
-cudaError_t launch_scale(const double *G, int nbin, int n_mock, double *C, cudaStream_t s);
-
 // ---- linear maps before the covariance (project.cu) ----
 // out[rows][n_s/f_s][n_mu/f_mu] = group sums of in[rows][n_s][n_mu] (int64)
 cudaError_t launch_rebin(const long long *in, long long rows, int n_s, int n_mu, int f_s, int f_mu, long long *out,
