@@ -287,9 +287,9 @@ int tpcf_multipole_matrix(int n_s, int n_mu, const int *ells, int n_ell, double 
  * symmetric matrix C[n][n] (device float64; only symmetric input is
  * meaningful), for checking that an LC covariance is positive definite
  * before it is inverted (Sect. 3.4).  Householder reduction to tridiagonal
- * form (one cluster of 8 blocks, the matrix in their shared memory up to
- * n = 472, in device memory above), then 32-way multisection on Sturm counts
- * taken on the continuants of T - x I (one warp per eigenvalue); absolute
+ * form (one cluster of 8 or 16 blocks, the matrix in their shared memory up
+ * to n = 628, in device memory above), then multisection on Sturm counts taken
+ * on the continuants of T - x I (one warp per eigenvalue); absolute
  * accuracy about n * 1e-16 * max|w|.
  * Needs 1 <= n <= 1024 (TPCF_ERR_ARG otherwise).
  *

@@ -104,6 +104,7 @@ __device__ __forceinline__ uint32_t cluster_rank()
 // before the barrier ahead of its reads after it
 __device__ __forceinline__ void cluster_sync_all()
 {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
@@ -193,169 +194,252 @@ __global__ void __cluster_dims__(TRI_CTAS, 1, 1) __launch_bounds__(TRI_THREADS)
     }
 }
 
-// a double in block `rank`'s shared memory at the offset of `p` in this block's
-__device__ __forceinline__ double ld_cluster(const double *p, uint32_t rank)
+// v into block `rank`'s shared memory at the offset of `p` in this block's
+__device__ __forceinline__ void st_cluster(double *p, uint32_t rank, double v)
 {
     const uint32_t la = (uint32_t)__cvta_generic_to_shared(p);
     uint32_t ra;
-    double v;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(la), "r"(rank));
-    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(ra) : "memory");
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(ra), "d"(v) : "memory");
+}
+
+// sum over the warp, in every lane
+__device__ __forceinline__ double warp_sum(double v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 
-// Shared-memory bytes of tridiag_smem_kernel for order n: block r's rows
-// (ceil(n / TRI_CTAS) of n doubles), v, w and the p of its rows.
-size_t tri_smem_bytes(int n)
+constexpr int TS_WARPS = 8;
+
+// Shared-memory bytes of tridiag_smem_kernel<C> for order n: block r's rows
+// (ceil(n / C) of n doubles) and six vectors.
+size_t tri_smem_bytes(int n, int C)
 {
-    const size_t R = ((size_t)n + TRI_CTAS - 1) / TRI_CTAS;
-    return (R * (size_t)n + 2 * (size_t)n + R) * sizeof(double);
+    const size_t R = ((size_t)n + C - 1) / C;
+    return (R * (size_t)n + 6 * (size_t)n) * sizeof(double);
 }
 
-// The same reduction with the matrix held in the cluster's shared memory
-// (orders whose rows fit: n <= 472): block r keeps the rows
-// i = r mod TRI_CTAS (local row t = global row r + TRI_CTAS t), reads row k
-// and the other blocks' p_i from their shared memory through the cluster's
-// address space, and updates its own rows in place; the input C is only read.
-__global__ void __cluster_dims__(TRI_CTAS, 1, 1) __launch_bounds__(TRI_THREADS)
-    tridiag_smem_kernel(const double *__restrict__ C, int n, double *__restrict__ d, double *__restrict__ e)
+// The same reduction with the matrix held in the shared memory of a cluster of
+// C blocks, block r with the rows i = r mod C, and one cluster barrier per
+// column.  What the other blocks need is written into their shared memory as
+// soon as it is known: p_i = beta (B v)_i by the row's owner, and the row that
+// the next column but one starts from.  At column k every block holds row k
+// (all updates applied: it gives the reflector) and, from its owner, row k + 1
+// as it was before column k; after the barrier, when all of p is there, every
+// block applies column k's update to row k + 1 itself, which is column k + 1's
+// start, while the owners update their rows.  Row i of B - v w^T - w v^T with
+// w = p - K v (K = beta p.v / 2) is b_i - v_i p - (p_i - 2 K v_i) v, so no
+// block forms w.  Warp 0 forms the next reflector while the other warps
+// update.  Inboxes and v are double-buffered: a block writes slot k mod 2
+// again only after a barrier that every block reaches past its last use.
+//
+// What bounds it: a column's chain of three reductions over a warp (0.26 us
+// each: 109 clocks per step), a square root and a division (0.33 us each) and
+// the barrier (0.18 us), and the float64 work, n^3 / C multiply-adds per SM at
+// two per clock.  n = 120: 759 -> 465 us against two barriers, reads of remote
+// rows and four block-wide reductions per column.
+template <int C>
+__global__ void __launch_bounds__(32 * TS_WARPS)
+    tridiag_smem_kernel(const double *__restrict__ A, int n, double *__restrict__ d, double *__restrict__ e)
 {
     extern __shared__ double sh[];
-    const int R = (n + TRI_CTAS - 1) / TRI_CTAS;
-    double *rows = sh;                    // [R][n]
-    double *v = rows + (size_t)R * n;     // [n]
-    double *w = v + n;                    // [n]
-    double *p = w + n;                    // [R], by local row
-    __shared__ double s_alpha, s_beta, s_k;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    const int R = (n + C - 1) / C;
+    double *rows = sh;                         // [R][n]
+    double *vb = rows + (size_t)R * n;         // [2][n] reflectors
+    double *pb = vb + 2 * (size_t)n;           // [2][n] inbox: p
+    double *xb = pb + 2 * (size_t)n;           // [2][n] inbox: row k + 1 before column k
+    __shared__ double s_beta[2], s_k;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = (int)cluster_rank();
-    const int nown = (n - rank + TRI_CTAS - 1) / TRI_CTAS;   // rows of this block (n > rank: n >= 3 here)
+    const int nown = (n - rank + C - 1) / C;   // rows of this block
     for (int idx = tid; idx < nown * n; idx += blockDim.x) {
         const int t = idx / n, j = idx % n;
-        rows[(size_t)t * n + j] = C[(size_t)(rank + TRI_CTAS * t) * n + j];
+        rows[(size_t)t * n + j] = A[(size_t)(rank + C * t) * n + j];
     }
-    cluster_sync_all();
-    for (int k = 0; k + 2 < n; k++) {
+    for (int j = tid; j < n; j += blockDim.x) xb[n + j] = A[(size_t)n + j];   // row 1
+
+    // one warp: the reflector of column k from row k, x(j) for j >= k
+    auto reflector = [&](int k, auto x) {
         const int m0 = k + 1;
-        const uint32_t ok = (uint32_t)(k % TRI_CTAS);      // the block that holds row k
-        const double *rk = rows + (size_t)(k / TRI_CTAS) * n;   // row k, at its offset in block ok
-        double ss = 0.0;
-        for (int i = m0 + 1 + tid; i < n; i += blockDim.x) {
-            const double x = ld_cluster(rk + i, ok);
-            v[i] = x;
-            ss = fma(x, x, ss);
+        double *v = vb + (k & 1) * (size_t)n;
+        double ss = 0.0, x0 = 0.0;
+        for (int j = m0 + lane; j < n; j += 32) {
+            const double xj = x(j);
+            v[j] = xj;
+            if (j == m0) x0 = xj; else ss = fma(xj, xj, ss);
         }
-        const double tail = block_sum(ss);
-        if (tid == 0) {
-            const double x0 = ld_cluster(rk + m0, ok);
-            if (tail == 0.0) {
-                s_alpha = x0;      // column already reduced: H = I
-                s_beta = 0.0;
-            } else {
+        const double xk = lane == 0 ? x(k) : 0.0;
+        const double tail = warp_sum(ss);
+        if (lane == 0) {
+            double alpha = x0, beta = 0.0;   // tail = 0: already reduced, H = I
+            if (tail != 0.0) {
                 const double nx = sqrt(fma(x0, x0, tail));
-                const double alpha = x0 > 0.0 ? -nx : nx;
+                alpha = x0 > 0.0 ? -nx : nx;
                 const double v0 = x0 - alpha;
-                s_alpha = alpha;
-                s_beta = 2.0 / fma(v0, v0, tail);   // 2 / (v.v)
+                beta = 2.0 / fma(v0, v0, tail);   // 2 / (v.v)
                 v[m0] = v0;
             }
-            if ((uint32_t)rank == ok) d[k] = rk[k];
-            if (rank == 0) e[k] = s_alpha;
+            s_beta[k & 1] = beta;
+            if (rank == 0) {
+                d[k] = xk;
+                e[k] = alpha;
+            }
         }
-        __syncthreads();
-        const double beta = s_beta;
-        if (beta == 0.0) continue;   // nothing written in this column: no barrier needed
-        // p_i = beta (B v)_i for this block's rows i >= m0, one warp per row
-        const int t0 = (m0 - rank + TRI_CTAS - 1) / TRI_CTAS > 0 ? (m0 - rank + TRI_CTAS - 1) / TRI_CTAS : 0;
-        for (int t = t0 + warp; t < nown; t += nw) {
-            const double *row = rows + (size_t)t * n;
-            double x = 0.0;
-            for (int j = m0 + lane; j < n; j += 32) x = fma(row[j], v[j], x);
-            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-            if (lane == 0) p[t] = beta * x;
+        __syncwarp();
+    };
+    if (warp == 0) reflector(0, [&](int j) { return A[j]; });
+    __syncthreads();
+    cluster_sync_all();   // every block has started: its shared memory may be written
+
+    for (int k = 0; k + 2 < n; k++) {
+        const int m0 = k + 1;
+        const double *v = vb + (k & 1) * (size_t)n;
+        double *p = pb + (k & 1) * (size_t)n;
+        const double beta = s_beta[k & 1];
+        const int t0 = (m0 - rank + C - 1) / C > 0 ? (m0 - rank + C - 1) / C : 0;
+        if (beta != 0.0) {
+            // p_i for this block's rows i >= m0, two rows per warp at a time
+            for (int t = t0 + 2 * warp; t < nown; t += 2 * TS_WARPS) {
+                const bool two = t + 1 < nown;
+                const double *r0 = rows + (size_t)t * n, *r1 = two ? r0 + n : r0;
+                double a0 = 0.0, a1 = 0.0;
+#pragma unroll 4
+                for (int j = m0 + lane; j < n; j += 32) {
+                    const double vj = v[j];
+                    a0 = fma(r0[j], vj, a0);
+                    a1 = fma(r1[j], vj, a1);
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+                    a1 += __shfl_xor_sync(0xffffffffu, a1, o);
+                }
+                if (lane < C) st_cluster(p + rank + C * t, (uint32_t)lane, beta * a0);
+                if (two && lane < C) st_cluster(p + rank + C * (t + 1), (uint32_t)lane, beta * a1);
+            }
         }
         cluster_sync_all();
-        double pv = 0.0;
-        for (int i = m0 + tid; i < n; i += blockDim.x) {
-            const double pi = ld_cluster(p + i / TRI_CTAS, (uint32_t)(i % TRI_CTAS));
-            w[i] = pi;
-            pv = fma(pi, v[i], pv);
+        double K = 0.0;
+        if (beta != 0.0) {
+            if (warp == 0) {
+                double pv = 0.0;
+#pragma unroll 4
+                for (int i = m0 + lane; i < n; i += 32) pv = fma(p[i], v[i], pv);
+                pv = warp_sum(pv);
+                if (lane == 0) s_k = 0.5 * beta * pv;
+            }
+            __syncthreads();
+            K = s_k;
         }
-        pv = block_sum(pv);
-        if (tid == 0) s_k = 0.5 * beta * pv;
+        if (warp == 0) {
+            // row k + 1 after this column's update: column k + 1's start
+            const double *y = xb + ((k + 1) & 1) * (size_t)n;
+            if (k + 3 < n) {
+                if (beta != 0.0) {
+                    const double vi = -v[m0], ui = -fma(-2.0 * K, v[m0], p[m0]);
+                    reflector(k + 1, [&](int j) { return fma(vi, p[j], fma(ui, v[j], y[j])); });
+                } else {
+                    reflector(k + 1, [&](int j) { return y[j]; });
+                }
+            } else if (rank == 0) {   // the last column: d and e of the remaining 2 x 2 block's first row
+                const double vi = -v[m0], ui = beta != 0.0 ? -fma(-2.0 * K, v[m0], p[m0]) : 0.0;
+                if (lane < 2) {
+                    const int j = n - 2 + lane;
+                    (lane ? e : d)[n - 2] = beta != 0.0 ? fma(vi, p[j], fma(ui, v[j], y[j])) : y[j];
+                }
+            }
+        } else {
+            // this block's rows i > k + 1, one warp per row; row k + 2 also goes to every block
+            for (int t = t0 + warp - 1; t < nown; t += TS_WARPS - 1) {
+                const int i = rank + C * t;
+                if (i == m0) continue;
+                double *r = rows + (size_t)t * n;
+                const double vi = beta != 0.0 ? -v[i] : 0.0, ui = beta != 0.0 ? -fma(-2.0 * K, v[i], p[i]) : 0.0;
+                double *out = xb + (k & 1) * (size_t)n;
+#pragma unroll 4
+                for (int j = m0 + lane; j < n; j += 32) {
+                    const double x = beta != 0.0 ? fma(vi, p[j], fma(ui, v[j], r[j])) : r[j];
+                    r[j] = x;
+                    if (i == k + 2 && k + 3 < n)
+#pragma unroll
+                        for (int q = 0; q < C; q++) st_cluster(out + j, (uint32_t)q, x);
+                }
+            }
+        }
         __syncthreads();
-        const double K = s_k;
-        for (int i = m0 + tid; i < n; i += blockDim.x) w[i] = fma(-K, v[i], w[i]);   // p becomes w
-        __syncthreads();
-        const int m = n - m0, nr = nown - t0;
-        for (int idx = tid; idx < nr * m; idx += blockDim.x) {
-            const int t = t0 + idx / m, j = m0 + idx % m, i = rank + TRI_CTAS * t;
-            double *x = rows + (size_t)t * n + j;
-            *x = fma(-v[i], w[j], fma(-w[i], v[j], *x));
-        }
-        cluster_sync_all();
     }
-    cluster_sync_all();   // no block leaves while another may still read its shared memory
-    if (tid == 0) {
-        const int i2 = n - 2, i1 = n - 1;
-        if (i2 % TRI_CTAS == rank) d[i2] = rows[(size_t)(i2 / TRI_CTAS) * n + i2];
-        if (i1 % TRI_CTAS == rank) {
-            e[i2] = rows[(size_t)(i1 / TRI_CTAS) * n + i2];
-            d[i1] = rows[(size_t)(i1 / TRI_CTAS) * n + i1];
-        }
-    }
+    cluster_sync_all();   // no block leaves while another may still write its shared memory
+    if ((n - 1) % C == rank && tid == 0) d[n - 1] = rows[(size_t)((n - 1) / C) * n + n - 1];
 }
 
-// Number of eigenvalues below x of the tridiagonal T = (d, e) scaled so that
-// its Gershgorin norm lies in [1, 2) (e2[i] = e[i]^2), without division: the
-// continuants p_i of T - x I (its leading principal minors, p_{-1} = 1,
-// p_i = (d_i - x) p_{i-1} - e2_{i-1} p_{i-2}) change sign exactly where the
-// ratios q_i = p_i / p_{i-1} of the Sturm sequence are negative, and each step
-// rounds like the ratio form's (one relative error on e2 p_{i-2}, one on the
-// result), so the count is that of a matrix within a few ulps of T.  A zero
-// p_i stands for the ratio -pivmin.  p_i and p_{i-1} are rescaled together by
-// a power of two (exactly) whenever p_i leaves [2^-300, 2^300]; with
-// |q_i| in [pivmin, 3 + 1 / pivmin] and pivmin = 2^-400 no step leaves the
-// range of normal doubles.  Three FP64 operations per step where the ratio
-// form needs a division (GB300's FP64 pipe is the bound).
-__device__ int sturm_count(const double *d, const double *e2, int n, double x)
+// The continuants p_i of T - x I (leading principal minors: p_{-1} = 1, p_i =
+// (d_i - x) p_{i-1} - e2_{i-1} p_{i-2}) of the tridiagonal T = (d, e) scaled so
+// that its norm lies in [1, 2): the number of sign changes is the number of
+// eigenvalues below x, without a division per step, and each step rounds like
+// the ratio form of the Sturm sequence, so the count is that of a matrix
+// within a few ulps of T.  t[i] = (d_i, e2_{i-1}), e2 at least 2^-120 (a
+// perturbation of T by 2^-60).  An exact zero becomes a tiny value of the
+// opposite sign of p_{i-1}, which no later comparison can tell from it.  The
+// pair (p_i, p_{i-1}) is rescaled by a power of two (exactly) every four
+// steps: its larger member changes by 2^-123 to 2^3 per step, so nothing leaves
+// the normal range in between.  Returns the count; (m, ex): the last continuant
+// as m 2^ex.
+__device__ __forceinline__ int sturm_count(const double2 *t, int n, double x, double &m, int &ex)
 {
-    constexpr double pivmin = 0x1p-400;
-    double pm = 1.0, p = d[0] - x;
-    if (p == 0.0) p = -pivmin;
-    int c = p < 0.0;
-    for (int i = 1; i < n; i++) {
-        double pn = fma(d[i] - x, p, -(e2[i - 1] * pm));
-        if (((__double2hiint(pn) & 0x7fffffff) | __double2loint(pn)) == 0) pn = -pivmin * p;
-        c += (__double2hiint(pn) ^ __double2hiint(p)) < 0;   // the signs differ
+    double pm = 0.0, p = 1.0;
+    int c = 0, shift = 0;
+    auto step = [&](double2 q) {
+        double pn = fma(q.x - x, p, -(q.y * pm));
+        const int hp = __double2hiint(p);
+        int hn = __double2hiint(pn);
+        if (((hn & 0x7fffffff) | __double2loint(pn)) == 0) {
+            hn = 0x01700000 | (~hp & (int)0x80000000);   // 2^-1000, sign opposite to p
+            pn = __hiloint2double(hn, 0);
+        }
+        c += (int)((uint32_t)(hn ^ hp) >> 31);
         pm = p;
         p = pn;
-        const int eb = (__double2hiint(p) >> 20) & 0x7ff;
-        if (eb > 1023 + 300 || eb < 1023 - 300) {
-            p = scalbn(p, 1023 - eb);
-            pm = scalbn(pm, 1023 - eb);
+    };
+    int i = 0;
+    for (; i + 4 <= n; i += 4) {
+        const double2 q0 = t[i], q1 = t[i + 1], q2 = t[i + 2], q3 = t[i + 3];
+        step(q0);
+        step(q1);
+        step(q2);
+        step(q3);
+        const int eb = max(__double2hiint(p) & 0x7ff00000, __double2hiint(pm) & 0x7ff00000) >> 20;
+        if (eb > 1023 + 200 || eb < 1023 - 200) {
+            const double f = __hiloint2double((2046 - eb) << 20, 0);
+            p *= f;
+            pm *= f;
+            shift += eb - 1023;
         }
     }
+    for (; i < n; i++) step(t[i]);
+    m = p;
+    ex = shift;
     return c;
 }
 
-// eigenvalue i (ascending) by multisection on the Sturm count, one warp per
-// eigenvalue: from the Gershgorin interval, each step the lanes j < 31 count
-// the eigenvalues below lo + (j + 1)(hi - lo) / 32 and the bracket becomes
-// the first of the 32 sub-intervals whose upper end counts more than i, so a
-// step gains 5 bits where bisection gains 1 (the FP64 Sturm counts are
-// spread over all SMs instead of one thread each); it stops when a step no
-// longer shrinks the bracket (a few ulps), at most 64 steps.  The block stages
-// T scaled by a power of two (exactly) to a norm in [1, 2) in shared memory.
-constexpr int EIG_WARPS = 2;   // eigenvalues per block
-
-__global__ void __launch_bounds__(32 * EIG_WARPS) multisect_kernel(const double *__restrict__ d,
-                                                                   const double *__restrict__ e, int n,
-                                                                   double *__restrict__ w)
+// eigenvalue i (ascending), one warp each, by multisection on the Sturm count
+// from the Gershgorin interval: every round the lanes' 31 points shrink the
+// bracket [lo, hi] (count(lo) <= i < count(hi)).  While the bracket holds
+// other eigenvalues the points divide it evenly (5 bits a round).  Once it
+// holds this one alone, the determinant changes sign in it, and sixteen of the
+// points close in geometrically on the secant's root (whose error falls with
+// the square of the bracket) while fifteen still divide it evenly: about
+// seven rounds instead of twelve.  Ends when the bracket is down to two of its
+// last places or a round no longer shrinks it.  The block stages T scaled by a
+// power of two (exactly) to a norm in [1, 2).  Bound by the float64 pipe and
+// the chain of n dependent multiply-adds per round; one warp per block, so
+// that no two share an SM while there are SMs left (n = 120: 361 -> 175 us).
+__global__ void __launch_bounds__(32) multisect_kernel(const double *__restrict__ d, const double *__restrict__ e,
+                                                       int n, double *__restrict__ w)
 {
-    extern __shared__ double sde[];
-    double *ds = sde, *e2s = sde + n;   // [n] each
-    const int lane = threadIdx.x & 31, i = blockIdx.x * EIG_WARPS + (threadIdx.x >> 5);
+    extern __shared__ double2 st[];   // [n]
+    const int lane = threadIdx.x & 31, i = blockIdx.x;
     double lo = INFINITY, hi = -INFINITY, nrm = 0.0;
     for (int k = lane; k < n; k += 32) {
         const double r = (k > 0 ? fabs(e[k - 1]) : 0.0) + (k + 1 < n ? fabs(e[k]) : 0.0);
@@ -368,33 +452,116 @@ __global__ void __launch_bounds__(32 * EIG_WARPS) multisect_kernel(const double 
         hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
         nrm = fmax(nrm, __shfl_xor_sync(0xffffffffu, nrm, o));
     }
-    const int ks = nrm > 0.0 ? ilogb(nrm) : 0;   // T / 2^ks has its norm in [1, 2)
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        ds[k] = scalbn(d[k], -ks);
-        const double ek = k + 1 < n ? scalbn(e[k], -ks) : 0.0;
-        e2s[k] = ek * ek;
+    if (nrm == 0.0) {   // T = 0
+        if (lane == 0) w[i] = 0.0;
+        return;
     }
-    __syncthreads();
-    if (i >= n) return;   // whole warps, after the block's last barrier
+    const int ks = ilogb(nrm);   // T / 2^ks has its norm in [1, 2)
+    for (int k = lane; k < n; k += 32) {
+        const double ek = k > 0 ? scalbn(e[k - 1], -ks) : 0.0;
+        st[k] = make_double2(scalbn(d[k], -ks), k > 0 ? fmax(ek * ek, 0x1p-120) : 0.0);
+    }
+    __syncwarp();
     const double pad = 4e-16 * n;
     lo = scalbn(lo, -ks) - pad;
     hi = scalbn(hi, -ks) + pad;
-    for (int it = 0; it < 64; it++) {
-        const double step = (hi - lo) * (1.0 / 32.0);
-        const double x = fmin(fma((double)(lane + 1), step, lo), hi);
-        const bool above = lane < 31 && sturm_count(ds, e2s, n, x) > i;
-        const unsigned mk = __ballot_sync(0xffffffffu, above);
-        const int f = mk ? __ffs(mk) - 1 : 31;   // sub-interval f: (x_{f-1}, x_f]
-        const double xf = __shfl_sync(0xffffffffu, x, f), xp = __shfl_sync(0xffffffffu, x, f > 0 ? f - 1 : 0);
-        const double nlo = f > 0 ? xp : lo, nhi = f < 31 ? xf : hi;
-        if (!(nlo > lo || nhi < hi)) break;
-        lo = nlo;
-        hi = nhi;
+    // Everything but the counts runs on the integer and FP32 pipes: a float64 operation holds a warp's issue for 64
+    // clocks.  Ends of the bracket by order-preserving integer keys; a point is lo + (hi - lo) frac with an FP32 frac.
+    auto key = [](double v) -> long long {
+        const long long b = __double_as_longlong(v);
+        return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+    };
+    auto expo = [](double v) -> int { return (__double2hiint(v) >> 20) & 0x7ff; };
+    const float geo = (lane & 1 ? 1.0f : -1.0f) * __int_as_float((127 - 5 - 2 * ((lane - 15) >> 1)) << 23);
+    int clo = 0, chi = n, exlo = 0, exhi = 0;   // counts and determinants at the bracket's ends
+    double mlo = 0.0, mhi = 0.0;                // 0: not known
+    for (int it = 0; it < 96; it++) {
+        const double h = hi - lo;
+        // done: the bracket is 2 last places of its ends, or empty
+        if (h <= 0.0 || expo(h) <= max(1023 - 320, max(expo(lo), expo(hi)) - 51)) break;
+        float frac = (float)(lane + 1) * (1.0f / 32.0f);
+        if (clo == i && chi == i + 1 && mlo != 0.0 && mhi != 0.0) {
+            if (lane < 15) {
+                frac = (float)(lane + 1) * (1.0f / 16.0f);
+            } else {   // the secant's root a / (a + b), a and b the determinants at lo and hi
+                const float fa = __int_as_float((__double2hiint(mlo) & 0xfffff) << 3 | 0x3f800000);
+                const float fb = __int_as_float((__double2hiint(mhi) & 0xfffff) << 3 | 0x3f800000);
+                const int dx = max(-60, min(60, expo(mhi) + exhi - expo(mlo) - exlo));
+                const float ratio = __fdividef(fb, fa) * __int_as_float((127 + dx) << 23);
+                frac = fminf(fmaxf(__fdividef(1.0f, 1.0f + ratio) + geo, 0.0f), 1.0f);
+            }
+        }
+        const double x = fma(h, (double)frac, lo);
+        double m;
+        int ex;
+        const int c = sturm_count(st, n, x, m, ex);
+        const bool above = c > i;
+        // the highest point that is not above and the lowest that is (lane 31's point takes part in neither)
+        const long long kx = key(x), none = 0x7fffffffffffffffll;
+        long long bl = lane < 31 && !above ? kx : -none, bh = lane < 31 && above ? kx : none;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            bl = max(bl, __shfl_xor_sync(0xffffffffu, bl, o));
+            bh = min(bh, __shfl_xor_sync(0xffffffffu, bh, o));
+        }
+        bool moved = false;
+        if (bl > key(lo)) {
+            const int l = __ffs(__ballot_sync(0xffffffffu, lane < 31 && !above && kx == bl)) - 1;
+            lo = __shfl_sync(0xffffffffu, x, l);
+            clo = __shfl_sync(0xffffffffu, c, l);
+            mlo = __shfl_sync(0xffffffffu, m, l);
+            exlo = __shfl_sync(0xffffffffu, ex, l);
+            moved = true;
+        }
+        if (bh < key(hi)) {
+            const int l = __ffs(__ballot_sync(0xffffffffu, lane < 31 && above && kx == bh)) - 1;
+            hi = __shfl_sync(0xffffffffu, x, l);
+            chi = __shfl_sync(0xffffffffu, c, l);
+            mhi = __shfl_sync(0xffffffffu, m, l);
+            exhi = __shfl_sync(0xffffffffu, ex, l);
+            moved = true;
+        }
+        if (!moved) break;
     }
     if (lane == 0) w[i] = scalbn(0.5 * (lo + hi), ks);
 }
 
 int blocks_for(size_t n, int threads) { return (int)std::max<size_t>(1, std::min<size_t>((n + threads - 1) / threads, 152 * 16)); }
+
+template <int C>
+cudaError_t launch_tridiag_smem(const double *A, int n, double *d, double *e, cudaStream_t s)
+{
+    const size_t sb = tri_smem_bytes(n, C);
+    cudaError_t err = cudaFuncSetAttribute(tridiag_smem_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb);
+    if (err == cudaSuccess && C > 8)
+        err = cudaFuncSetAttribute(tridiag_smem_kernel<C>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (err != cudaSuccess) return err;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(C);
+    cfg.blockDim = dim3(32 * TS_WARPS);
+    cfg.dynamicSmemBytes = sb;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, tridiag_smem_kernel<C>, A, n, d, e);
+}
+
+// The cluster size of the shared-memory reduction for order n: 16 blocks (an
+// opt-in size) from n = 96, below which 8 do as well, else 8; 0 when the matrix
+// does not fit (n > 628).  Whole call with 16 / with 8 / before: n = 96
+// 497 / 497 / 874 us, 120 675 / 698 / 1134, 200 1224 / 1434 / 2125, 420 4132 /
+// 5930 / 6794, 600 8458 / - / 16750.
+int pick_cluster(int n)
+{
+    constexpr size_t room = (size_t)226 << 10;
+    if (n >= 96 && tri_smem_bytes(n, 16) <= room) return 16;
+    return tri_smem_bytes(n, 8) <= room ? 8 : 0;
+}
 
 }  // namespace
 
@@ -430,19 +597,20 @@ cudaError_t launch_eigvalsh(const double *C, int n, double *work, double *w, cud
 {
     double *a = work, *d = work + (size_t)n * n, *e = d + n, *pg = e + n;
     cudaError_t err;
-    const size_t sb = tri_smem_bytes(n);
-    if (n >= 3 && sb <= (size_t)(226 << 10)) {
-        // the matrix fits in the cluster's shared memory
-        err = cudaFuncSetAttribute(tridiag_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb);
+    int cl = 0;   // blocks of the cluster whose shared memory holds the matrix; 0: it does not fit
+    if (n >= 3) cl = pick_cluster(n);
+    if (cl == 16) {
+        err = launch_tridiag_smem<16>(C, n, d, e, s);
         if (err != cudaSuccess) return err;
-        tridiag_smem_kernel<<<TRI_CTAS, TRI_THREADS, sb, s>>>(C, n, d, e);
+    } else if (cl == 8) {
+        err = launch_tridiag_smem<8>(C, n, d, e, s);
+        if (err != cudaSuccess) return err;
     } else {
         err = cudaMemcpyAsync(a, C, (size_t)n * n * sizeof(double), cudaMemcpyDeviceToDevice, s);
         if (err != cudaSuccess) return err;
         tridiag_kernel<<<TRI_CTAS, TRI_THREADS, 2 * (size_t)n * sizeof(double), s>>>(a, n, d, e, pg);
     }
-    multisect_kernel<<<(n + EIG_WARPS - 1) / EIG_WARPS, 32 * EIG_WARPS, 2 * (size_t)n * sizeof(double), s>>>(d, e,
-                                                                                                          n, w);
+    multisect_kernel<<<n, 32, (size_t)n * sizeof(double2), s>>>(d, e, n, w);
     return cudaGetLastError();
 }
 
