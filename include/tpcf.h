@@ -404,8 +404,9 @@ int tpcf_set_cell_subdiv(tpcf_ctx *ctx, int subdiv);
  *                        time candidates on a few of the mocks (all of them
  *                        below 2e6 points) and keep the fastest: the pair
  *                        counter (both, under TPCF_KERNEL_AUTO), the mesh
- *                        subdivision {2, 3, 4} and the work-unit size
- *                        {64, 128}, then fewer blocks per SM for the winner
+ *                        subdivision {2, 3, 4} (1 too for sparse catalogues)
+ *                        and the work-unit size {64, 128}, then fewer blocks
+ *                        per SM for the winner
  *                        (cached per context, keyed by the binning, the
  *                        classes log2 of the mean catalogue size and of the
  *                        number of mocks, and the device's name, SM count and

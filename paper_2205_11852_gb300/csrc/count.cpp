@@ -138,7 +138,7 @@ int prepare(tpcf_ctx *ctx, const tpcf_mock *mocks, int n_mock, const tpcf_binnin
             cudaGetLastError();
             sm_sm = 0;
         }
-        if (sm_sm > 0 && build_direct(*binning, S.pl, sm_sm, sm_blk, resv, max_cat, S.dp)) {
+        if (sm_sm > 0 && build_direct(*binning, S.pl, sm_sm, sm_blk, resv, max_cat, cfg.group, S.dp)) {
             S.direct = true;
             S.chunk = std::min(S.chunk, DIRECT_ACHUNK);
         }
@@ -195,6 +195,7 @@ int prepare(tpcf_ctx *ctx, const tpcf_mock *mocks, int n_mock, const tpcf_binnin
                 S.terms.push_back(Term{cr + i, cr + i, 1, 0, (long long *)rr + ((size_t)m * M + i) * nbin});
         }
     }
+    bool even = true;   // no mock costs much more than the mean
     // longest first: mocks in decreasing order of their pair count (the sum over their terms of n_a n_b,
     // or n (n - 1) / 2 for an auto count), each mock's terms kept together (its catalogues stay in L2), so
     // that the units claimed last, at the end of a launch, belong to the cheapest mocks
@@ -209,6 +210,9 @@ int prepare(tpcf_ctx *ctx, const tpcf_mock *mocks, int n_mock, const tpcf_binnin
         std::vector<int> order(n_mock);
         for (int m = 0; m < n_mock; m++) order[m] = m;
         std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return mc[x] > mc[y]; });
+        double all = 0.0;
+        for (double c : mc) all += c;
+        even = n_mock > 0 && mc[order[0]] * n_mock <= 1.25 * all;
         std::vector<Term> sorted;
         sorted.reserve(S.terms.size());
         for (int m : order)
@@ -225,11 +229,12 @@ int prepare(tpcf_ctx *ctx, const tpcf_mock *mocks, int n_mock, const tpcf_binnin
 
     S.ncc = S.cats.size() * (size_t)prm.n_cells + 1;
     if (S.ncc >= (1ull << 32)) return fail(ctx, TPCF_ERR_RANGE, "too many catalogues x cells");
-    S.ntc = S.terms.size() * (size_t)prm.n_cells + 1;
+    const size_t n_groups = S.direct ? S.dp.n_groups : prm.n_cells;
+    S.ntc = S.terms.size() * n_groups + 1;
     if (S.ntc >= (1ull << 32)) return fail(ctx, TPCF_ERR_RANGE, "too many terms x cells");
     for (const Term &t : S.terms) {
         const unsigned long long n = S.cats[t.cat_a].n;
-        S.units_bound += n / S.chunk + std::min<unsigned long long>(n, prm.n_cells) + 1;
+        S.units_bound += n / S.chunk + std::min<unsigned long long>(n, n_groups) + 1;
     }
     S.tmp_n = std::max(scan_tmp_elems(S.ncc), scan_tmp_elems(S.ntc));
 
@@ -290,16 +295,16 @@ int prepare(tpcf_ctx *ctx, const tpcf_mock *mocks, int n_mock, const tpcf_binnin
         if (occ < 1) return fail(ctx, TPCF_ERR_CUDA, "the direct pair counter does not fit on an SM");
         S.smem = S.dp.smem;
         S.blocks = ctx->n_sm * (cfg.bps > 0 ? std::min(cfg.bps, occ) : occ);
-        // units per block claim, at most 2^30 pairs per counter: about eight claims per block in the
-        // batched launch; in the one-launch-per-term mode one claim per block of the term's share (every
-        // claim ends in a block barrier, which a launch of one term cannot amortise)
+        // units per block claim (claims shrink toward the end of the launch): in the batched launch a quarter of a
+        // block's share, or an eighth where the mocks, in decreasing order of cost, are uneven (a first claim of a
+        // quarter from the largest mocks left 0.34 of the warps' time idle on cut-sky mocks of 50 000 to 400 000
+        // points, an eighth 0.0015); in the one-launch-per-term mode a block's share of the term
         const unsigned long long by_work =
             mode == TPCF_PER_LAUNCH
                 ? std::max<unsigned long long>(1, (S.units_bound / std::max<size_t>(1, S.terms.size()) + S.blocks - 1) /
                                                       (unsigned long long)S.blocks)
-                : std::max<unsigned long long>(1, S.units_bound / (8ull * S.blocks));
-        const unsigned long long by_wrap = std::max<unsigned long long>(1, (1ull << 30) / S.dp.unit_pair_bound);
-        S.claim_units = (int)std::min<unsigned long long>({by_work, by_wrap, 4096ull});
+                : std::max<unsigned long long>(1, S.units_bound / ((even ? 4ull : 8ull) * (unsigned long long)S.blocks));
+        S.claim_units = (int)std::min<unsigned long long>(by_work, 4096ull);
         return TPCF_OK;
     }
     S.smem = paircount_smem_bytes(prm, 8);
@@ -374,9 +379,10 @@ int enqueue(tpcf_ctx *ctx, const Setup &S, int mode, cudaStream_t s, void *small
     if (mode == TPCF_BATCHED || S.direct) {
         // the work-unit list (the direct counter uses it in both modes)
         CK(cudaMemsetAsync(uc + (S.ntc - 1), 0, 4, s));
-        CK(launch_unit_count(d_terms, n_terms, d_cats, prm.n_cells, cs, S.chunk, uc, s));
+        const int G = S.direct ? S.dp.G : 1;
+        CK(launch_unit_count(d_terms, n_terms, prm.n_c, G, cs, S.chunk, uc, s));
         CK(launch_scan_u32(uc, ust, S.ntc, tmp, S.tmp_n, s));
-        CK(launch_unit_fill(d_terms, n_terms, d_cats, prm.n_cells, cs, S.chunk, ust, (Unit *)S.units, s));
+        CK(launch_unit_fill(d_terms, n_terms, prm.n_c, G, cs, S.chunk, ust, (Unit *)S.units, s));
         CK(cudaMemsetAsync(S.claim, 0, 4 * (S.terms.size() + 1), s));
         kernels += 5;
     }
@@ -387,8 +393,8 @@ int enqueue(tpcf_ctx *ctx, const Setup &S, int mode, cudaStream_t s, void *small
         if (ev0) CK(cudaEventRecordWithFlags(ev0, s, external ? cudaEventRecordExternal : cudaEventRecordDefault));
         if (S.direct) {
             L.chunk = S.claim_units;
-            CK(launch_pairdirect(prm, S.dp, mesh, d_terms, (const Unit *)S.units, ust + (S.ntc - 1),
-                                 (unsigned *)S.claim, ctx->stats, L, s));
+            CK(launch_pairdirect(prm, S.dp, mesh, d_terms, (const Unit *)S.units, ust, ust + (S.ntc - 1),
+                                 (unsigned *)S.claim, ctx->stats, ctx->status, L, s));
         } else {
             CK(launch_paircount(prm, mesh, d_terms, d_cats, (const Unit *)S.units, ust + (S.ntc - 1),
                                 (unsigned *)S.claim, d_tab, ctx->stats, ctx->status, L, s));
@@ -407,8 +413,8 @@ int enqueue(tpcf_ctx *ctx, const Setup &S, int mode, cudaStream_t s, void *small
                 // block barriers (each waits for the block's slowest warp) fall in one launch
                 L.blocks = S.blocks;
                 L.chunk = std::max(1, S.claim_units);
-                CK(launch_pairdirect(prm, S.dp, mesh, d_terms, (const Unit *)S.units, ust + (S.ntc - 1),
-                                     (unsigned *)S.claim + 1 + t, ctx->stats, L, s));
+                CK(launch_pairdirect(prm, S.dp, mesh, d_terms, (const Unit *)S.units, ust, ust + (S.ntc - 1),
+                                     (unsigned *)S.claim + 1 + t, ctx->stats, ctx->status, L, s));
             } else {
                 L.blocks = std::min(S.blocks, prm.n_cells);   // blocks stride over the cells
                 CK(launch_paircount(prm, mesh, d_terms, d_cats, nullptr, nullptr, nullptr, d_tab, ctx->stats,
@@ -578,8 +584,9 @@ int run_direct(tpcf_ctx *ctx, const Setup &S, int mode, cudaStream_t s, int slot
 // Autotuner: times one batched count of the first few mocks per candidate
 // (at least 6, and all the mocks of a workload under 2e6 points).
 // Stage 1: pair counter (both, when the context leaves the choice to the
-// library) x mesh subdivision {2, 3, 4} x unit size {64, 128} (the direct
-// counter's unit is fixed at 64 a-points).  Stage 2, for the winner: fewer
+// library) x mesh subdivision {2, 3, 4}, and 1 for sparse catalogues, x unit
+// size {64, 128} (the direct counter's unit is fixed at 64 a-points), then units
+// of two cells for the direct counter on sparse catalogues.  Stage 2, for the winner: fewer
 // blocks per SM than fit (the persistent grid's occupancy).  Each candidate
 // is timed twice (six times when a run takes under 2 ms) and its fastest run
 // kept.
@@ -599,8 +606,10 @@ int autotune(tpcf_ctx *ctx, const tpcf_mock *mocks, int n_mock, const tpcf_binni
             n_try = std::max(n_try, m + 1);
         }
     }
-    static const int subdivs[] = {2, 3, 4};
     static const int chunks[] = {64, 128};
+    std::vector<int> subdivs = {2, 3, 4};
+    double per_cell = 0.0;   // mean points per catalogue and cell of the last prepared trial
+
     std::vector<int> kernels;
     if (ctx->kernel_pref == TPCF_KERNEL_AUTO) kernels = {TPCF_KERNEL_GENERAL, TPCF_KERNEL_DIRECT};
     else kernels = {ctx->kernel_pref};
@@ -610,6 +619,7 @@ int autotune(tpcf_ctx *ctx, const tpcf_mock *mocks, int n_mock, const tpcf_binni
     float best_ms = 1e30f;
     int rc = TPCF_OK;
     int best_occ = 0;
+    double best_per_cell = 0.0;
     // time candidate c; rc != 0 stops the search, a mesh or counter that does not fit is skipped
     auto trial = [&](const Tuned &c, int &occ_out) -> float {
         Setup S;
@@ -619,6 +629,7 @@ int autotune(tpcf_ctx *ctx, const tpcf_mock *mocks, int n_mock, const tpcf_binni
         }
         if (c.kernel == TPCF_KERNEL_DIRECT && !S.direct) return 1e30f;   // the general counter's timing is its own
         occ_out = S.blocks / std::max(1, ctx->n_sm);
+        per_cell = (double)S.NT / ((double)std::max<size_t>(1, S.cats.size()) * (double)S.pl.prm.n_cells);
         float ms = 1e30f;
         // two runs, six when they are short (launch latency makes those noisy)
         for (int rep = 0; rep < (rep >= 2 && ms < 2.0f ? 6 : 2) && rc == TPCF_OK; rep++) {
@@ -633,6 +644,22 @@ int autotune(tpcf_ctx *ctx, const tpcf_mock *mocks, int n_mock, const tpcf_binni
         }
         return ms;
     };
+    {
+        // cells as wide as the last edge (subdivision 1) where they hold 16 points or more but those of subdivision
+        // 2 fewer: a unit of few points spends its time on set-up (16 mocks of 4000 points, 32 a cell at
+        // subdivision 1 and five at 2: 0.23 ms against 0.36, and 0.30 with two cells per unit)
+        Setup S1, S2;
+        Tuned c;
+        c.kernel = TPCF_KERNEL_GENERAL;
+        c.subdiv = 1;
+        if (prepare(ctx, mocks, n_try, binning, terms, dd, dr, rr, TPCF_BATCHED, c, S1) == TPCF_OK && S1.NT > 0) {
+            c.subdiv = 2;
+            if (prepare(ctx, mocks, n_try, binning, terms, dd, dr, rr, TPCF_BATCHED, c, S2) == TPCF_OK) {
+                const double n = (double)S1.NT / (double)std::max<size_t>(1, S1.cats.size());
+                if (n >= 16.0 * S1.pl.prm.n_cells && n < 16.0 * S2.pl.prm.n_cells) subdivs.insert(subdivs.begin(), 1);
+            }
+        }
+    }
     for (int kern : kernels)
         for (int sd : subdivs)
             for (int ch : chunks) {
@@ -648,8 +675,26 @@ int autotune(tpcf_ctx *ctx, const tpcf_mock *mocks, int n_mock, const tpcf_binni
                     best_ms = ms;
                     best = c;
                     best_occ = occ;
+                    best_per_cell = per_cell;
                 }
             }
+    // units of two cells, where the winner's units hold few points
+    if (best.kernel == TPCF_KERNEL_DIRECT && best_per_cell < 16.0)
+        for (int sd : subdivs) {
+            Tuned c;
+            c.subdiv = sd;
+            c.chunk = chunks[0];
+            c.kernel = TPCF_KERNEL_DIRECT;
+            c.group = 2;
+            int occ = 0;
+            const float ms = trial(c, occ);
+            if (rc) goto done;
+            if (ms < best_ms) {
+                best_ms = ms;
+                best = c;
+                best_occ = occ;
+            }
+        }
     for (int bps = best_occ - 1; bps >= 1 && bps >= best_occ - 2; bps--) {
         Tuned c = best;
         c.bps = bps;

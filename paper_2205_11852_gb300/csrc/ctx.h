@@ -42,6 +42,7 @@ struct Tuned {
     int chunk = 256;
     int kernel = -1;   // TPCF_KERNEL_*; -1: the context's preference
     int bps = 0;       // blocks per SM of the pair counter; 0: as many as fit
+    int group = 1;     // direct counter: cells along x that share a unit
 };
 
 }  // namespace tpcf

@@ -198,30 +198,40 @@ __global__ void __launch_bounds__(SCAN_THREADS) tile_scan_kernel(const uint32_t 
 
 // ---- work units ----
 
-__global__ void unit_count_kernel(const Term *__restrict__ terms, int n_terms, const Cat *__restrict__ cats,
-                                  int n_cells, const uint32_t *__restrict__ cellstart, int chunk,
-                                  uint32_t *__restrict__ ucount)
+// a-points [s0, s1) of group g (G consecutive cells along x, fewer at a row's end) of term t; returns its first cell
+__device__ __forceinline__ int group_range(const Term &t, uint32_t g, uint32_t n_c, uint32_t G, uint32_t gpr,
+                                           const uint32_t *cellstart, uint32_t &s0, uint32_t &s1)
 {
-    const size_t total = (size_t)n_terms * n_cells;
+    const uint32_t row = g / gpr, x = (g - row * gpr) * G, cell = row * n_c + x;
+    const size_t gk = (size_t)t.cat_a * n_c * n_c * n_c + cell;
+    s0 = cellstart[gk];
+    s1 = cellstart[gk + min(G, n_c - x)];
+    return (int)cell;
+}
+
+__global__ void unit_count_kernel(const Term *__restrict__ terms, int n_terms, int n_c, int G, int gpr,
+                                  const uint32_t *__restrict__ cellstart, int chunk, uint32_t *__restrict__ ucount)
+{
+    const size_t ng = (size_t)n_c * n_c * gpr, total = (size_t)n_terms * ng;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int t = (int)(i / n_cells), cell = (int)(i % n_cells);
-        const size_t gk = (size_t)terms[t].cat_a * n_cells + cell;
-        const uint32_t n = cellstart[gk + 1] - cellstart[gk];
-        ucount[i] = (n + chunk - 1) / chunk;
+        uint32_t s0, s1;
+        group_range(terms[i / ng], (uint32_t)(i % ng), (uint32_t)n_c, (uint32_t)G, (uint32_t)gpr, cellstart, s0, s1);
+        ucount[i] = (s1 - s0 + chunk - 1) / chunk;
     }
 }
 
-__global__ void unit_fill_kernel(const Term *__restrict__ terms, int n_terms, const Cat *__restrict__ cats,
-                                 int n_cells, const uint32_t *__restrict__ cellstart, int chunk,
+__global__ void unit_fill_kernel(const Term *__restrict__ terms, int n_terms, int n_c, int G, int gpr,
+                                 const uint32_t *__restrict__ cellstart, int chunk,
                                  const uint32_t *__restrict__ ustart, Unit *__restrict__ units)
 {
-    const size_t total = (size_t)n_terms * n_cells;
+    const size_t ng = (size_t)n_c * n_c * gpr, total = (size_t)n_terms * ng;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const uint32_t u0 = ustart[i], u1 = ustart[i + 1];
         if (u0 == u1) continue;
-        const int t = (int)(i / n_cells), cell = (int)(i % n_cells);
-        const size_t gk = (size_t)terms[t].cat_a * n_cells + cell;
-        const uint32_t s0 = cellstart[gk], s1 = cellstart[gk + 1];
+        const int t = (int)(i / ng);
+        uint32_t s0, s1;
+        const int cell = group_range(terms[t], (uint32_t)(i % ng), (uint32_t)n_c, (uint32_t)G, (uint32_t)gpr,
+                                     cellstart, s0, s1);
         for (uint32_t j = 0; j < u1 - u0; j++) {
             Unit u;
             u.term = t;
@@ -291,22 +301,23 @@ cudaError_t launch_scatter(const Cat *cats, int n_cat, uint32_t max_n, const Cou
     return cudaGetLastError();
 }
 
-cudaError_t launch_unit_count(const Term *terms, int n_terms, const Cat *cats, int n_cells,
-                              const uint32_t *cellstart, int chunk, uint32_t *ucount, cudaStream_t s)
+cudaError_t launch_unit_count(const Term *terms, int n_terms, int n_c, int G, const uint32_t *cellstart, int chunk,
+                              uint32_t *ucount, cudaStream_t s)
 {
-    const size_t total = (size_t)n_terms * n_cells;
-    unit_count_kernel<<<grid_for(total, 256, 152 * 32), 256, 0, s>>>(terms, n_terms, cats, n_cells, cellstart,
-                                                                      chunk, ucount);
+    const int gpr = (n_c + G - 1) / G;
+    const size_t total = (size_t)n_terms * n_c * n_c * gpr;
+    unit_count_kernel<<<grid_for(total, 256, 152 * 32), 256, 0, s>>>(terms, n_terms, n_c, G, gpr, cellstart, chunk,
+                                                                      ucount);
     return cudaGetLastError();
 }
 
-cudaError_t launch_unit_fill(const Term *terms, int n_terms, const Cat *cats, int n_cells,
-                             const uint32_t *cellstart, int chunk, const uint32_t *ustart, Unit *units,
-                             cudaStream_t s)
+cudaError_t launch_unit_fill(const Term *terms, int n_terms, int n_c, int G, const uint32_t *cellstart, int chunk,
+                             const uint32_t *ustart, Unit *units, cudaStream_t s)
 {
-    const size_t total = (size_t)n_terms * n_cells;
-    unit_fill_kernel<<<grid_for(total, 256, 152 * 32), 256, 0, s>>>(terms, n_terms, cats, n_cells, cellstart,
-                                                                     chunk, ustart, units);
+    const int gpr = (n_c + G - 1) / G;
+    const size_t total = (size_t)n_terms * n_c * n_c * gpr;
+    unit_fill_kernel<<<grid_for(total, 256, 152 * 32), 256, 0, s>>>(terms, n_terms, n_c, G, gpr, cellstart, chunk,
+                                                                     ustart, units);
     return cudaGetLastError();
 }
 

@@ -29,6 +29,7 @@ __device__ __noinline__ int exact_bin(const CountParams &prm, const unsigned lon
     const int n_s = prm.n_s;
     if (D2 < T[0] || D2 >= T[n_s]) return -1;
     int lo = 0, hi = n_s - 1;        // largest k with T[k] <= D2
+#pragma unroll 1
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (T[mid] <= D2) lo = mid; else hi = mid - 1;
@@ -57,6 +58,7 @@ __device__ __noinline__ int exact_bin(const CountParams &prm, const unsigned lon
         if (den != 0) {
             const u128 lhs = (u128)(unsigned)(n_mu * n_mu) * num;
             j = n_mu - 1;
+#pragma unroll 1
             while (j > 0 && lhs < (u128)(unsigned)(j * j) * den) j--;
         }
     }

@@ -4,16 +4,20 @@
 // line of sight from the observer to the pair's midpoint (cut-sky mocks).
 //
 // Work decomposition.  A unit is a chunk of at most 64 sorted points of one
-// mesh cell A, paired with the neighbourhood of A in catalogue b.  Each warp
+// mesh cell A, or of a few cells in a row along x where the cells hold few
+// points, paired with the neighbourhood of A in catalogue b.  Each warp
 // owns a unit on its own: it stages the a-chunk in its region of shared
 // memory, streams the b-points of the neighbourhood (the self cell of an
 // auto count as it is, every other neighbour cell through a filter that
 // keeps a point only if its distance to the a-chunk's bounding box is below
 // the last edge) into its own buffer, and counts every full tile of 128
 // b-points (4 per lane) against the a-chunk as soon as it is there.  The
-// warps of a block share one histogram, so a block works through a chunk of
-// consecutive units of one term at a time (units are ordered by term); block
-// barriers come only between such chunks.
+// warps of a block share one to four histogram tables, one per term, and pass
+// from one term to the next without waiting for each other (see
+// pairdirect_kernel).  The code that few units need (locks, drains, rechecks)
+// keeps its loops rolled: with warps at different places the instruction cache
+// is what a larger kernel pays with (104 KB of code instead of 67: 4 % on cut-sky
+// mocks, 13 % on small ones).
 //
 // Arithmetic.  Coordinates are exact integer offsets from A's lower corner,
 // converted once to FP32 in units of one s bin, so the s bin of a pair is
@@ -40,9 +44,9 @@
 // Histogram.  R copies of a (n_s + 1) x C table of 32-bit counters, lane l
 // adding to copy l mod R, so the 32 adds of a warp fall in distinct banks
 // (R = 32) or at most two per bank (R = 16).  mu is binned by sign, C =
-// 2 n_mu + 2 columns from -n_mu - 1 to n_mu, and folded to |mu| when the
-// table is drained into the term's int64 histogram: when the block moves to
-// another term, or before its 32-bit counters could wrap.
+// 2 n_mu + 2 columns from -n_mu - 1 to n_mu, and folded to |mu| when a table is
+// drained into the term's int64 histogram: when the block's last warp leaves
+// the term, or before its 32-bit counters could wrap.
 #include "pair_device.cuh"
 
 namespace tpcf {
@@ -63,27 +67,42 @@ static_assert(DIRECT_ACHUNK % 32 == 0 && DIRECT_ACHUNK <= 64, "a-chunk load: two
 
 __host__ __device__ constexpr uint32_t al16(uint32_t x) { return (x + 15u) & ~15u; }
 
-// Shared memory: the block's histogram, T, misc words, then one region per
-// warp: a-records (3 float4 per a-point), the b buffer (float4: x, y, z in
+// How a block's warps share its work and its tables.  `claim` and `n_used`
+// change by atomics; the rest is read and written under `lock` (taken by one
+// lane of a warp for a few instructions).
+constexpr int MAX_NT = DIRECT_TABLES;
+struct Sched {
+    unsigned long long claim;   // the block's claim: next unit (low word; may pass the end) and end (high word)
+    unsigned n_used[MAX_NT];    // units taken for a table since it was last empty
+    unsigned lock;
+    int term[MAX_NT];           // the term a table counts, or FREE, or DRAINING
+    unsigned ref[MAX_NT];       // warps adding to a table
+};
+constexpr int FREE = -1, DRAINING = -2;
+
+// Shared memory: the block's one or two tables, T, the schedule, then one
+// region per warp: a-records (3 float4 per a-point), the b buffer (float4: x, y, z in
 // bins and the b index), the unit's runs (first index, offset in the
 // concatenation) and the recheck list.
 struct DOff {
-    uint32_t hist, T, misc, warp0, wstride;
-    uint32_t arec, buf, runs, xl;   // offsets inside a warp's region
+    uint32_t hist, hstride, T, misc, warp0, wstride;
+    uint32_t arec, buf, runs, xl, st;   // offsets inside a warp's region
     uint32_t end;
 };
-__host__ __device__ inline DOff d_off(int n_s, int n_rows, int R, int C, int W)
+__host__ __device__ inline DOff d_off(int n_s, int n_rows, int R, int C, int NT, int W)
 {
     DOff o;
     o.hist = 0;
-    o.T = al16(4u * (uint32_t)((n_s + 1) * C * R));
+    o.hstride = al16(4u * (uint32_t)((n_s + 1) * C * R));
+    o.T = o.hstride * (uint32_t)NT;
     o.misc = al16(o.T + 8u * (uint32_t)(n_s + 1));
-    o.warp0 = o.misc + 64u;
+    o.warp0 = o.misc + al16((uint32_t)sizeof(Sched));
     o.arec = 0;
     o.buf = o.arec + 48u * DIRECT_ACHUNK;
     o.runs = o.buf + 16u * BUF;
     o.xl = al16(o.runs + 8u * (uint32_t)(2 * n_rows + 1));
-    o.wstride = al16(o.xl + 8u * XCAP);
+    o.st = al16(o.xl + 8u * XCAP);
+    o.wstride = o.st + 48u;
     o.end = o.warp0 + o.wstride * (uint32_t)W;
     return o;
 }
@@ -107,9 +126,9 @@ struct ARec {
 // and LS = LT + log2(C), so that the row and column strides are shifts.
 template <int R, int LOGC>
 struct Sh {
-    static constexpr int LT = R == 32 ? 7 : (R == 16 ? 6 : -1);
+    static constexpr int LT = R == 32 ? 7 : (R == 16 ? 6 : (R == 8 ? 5 : -1));
     static constexpr int LS = LT + LOGC;
-    static_assert(LT > 0, "R is 16 or 32");
+    static_assert(LT > 0, "R is 8, 16 or 32");
 };
 
 __device__ __forceinline__ uint64_t u64of(float2 v) { return *reinterpret_cast<uint64_t *>(&v); }
@@ -492,11 +511,30 @@ __device__ __forceinline__ bool apoint(const float2 (&BX)[NQ], const float2 (&BY
 #undef PM_RED
 #undef PM_HEAD
 
-// Per-lane histogram address constants (see Sh).
+// Kl of the warp's table (see Sh), the histogram base (shared address) + 4
+// (lane mod R) and this lane's word in the spare last row.
+template <bool MU, int R, int LOGC>
 struct Addr {
+    static constexpr int LS = Sh<R, LOGC>::LS, LT = Sh<R, LOGC>::LT;
     uint32_t Kl;
-    uint32_t hb;      // histogram base (shared address) + 4 (lane mod R)
-    uint32_t dump;    // this lane's word in the spare last row
+    __device__ __forceinline__ static uint32_t shift(const DirectParams &dp)
+    {
+        return MU ? ((uint32_t)dp.CO << LT) - (MAG_S_BITS << LS) - (MAG_T_BITS << LT) : 0u - (MAG_S_BITS << LS);
+    }
+    __device__ __forceinline__ uint32_t hb(const DirectParams &dp) const { return Kl - shift(dp); }
+    __device__ __forceinline__ uint32_t dump(const CountParams &prm, const DirectParams &dp) const
+    {
+        return hb(dp) + ((uint32_t)prm.n_s << LS);
+    }
+};
+
+// What a warp keeps from unit to unit, in shared memory (the registers belong
+// to the tiles): counters for the launch's statistics, its table, the table's
+// term and that term's units [t_lo, t_hi).
+struct WarpState {
+    unsigned long long n_cand, n_exact, binned, t_start;
+    int tab, term;
+    uint32_t t_lo, t_hi;
 };
 
 // A warp's shared-memory region and its pending exact rechecks.
@@ -505,6 +543,7 @@ struct WarpMem {
     float4 *buf;      // b buffer: x, y, z in bins and the b index
     uint2 *runs;      // the unit's runs: (first b index, offset in their concatenation)
     uint2 *xl;        // pairs (a index, b index) awaiting the exact recheck
+    WarpState *st;
 };
 
 template <bool MID>
@@ -523,18 +562,19 @@ __device__ __forceinline__ ARec load_a(const float4 *arec, uint32_t ai)
 
 __device__ __forceinline__ void xl_put(uint2 *xl, uint32_t i, uint32_t ia, uint32_t ib) { xl[i] = make_uint2(ia, ib); }
 
-// exact recheck of the n listed pairs, one per lane; returns the number rechecked by this lane
+// exact recheck of the n listed pairs, one per lane
 template <bool MU, int R, int LOGC>
-__device__ __forceinline__ uint32_t recheck(const CountParams &prm, const DirectParams &dp, const Mesh &m,
-                                            const unsigned long long *T, const uint2 *xl, uint32_t n, uint32_t hb,
-                                            int lane)
+__device__ __forceinline__ void recheck(const CountParams &prm, const DirectParams &dp, const Mesh &m,
+                                        const unsigned long long *T, const WarpMem &wm, uint32_t n, uint32_t hb,
+                                        int lane)
 {
     __syncwarp();
-    uint32_t cnt = 0;
+    const uint2 *xl = wm.xl;
+    if (lane == 0) wm.st->n_exact += n;
+#pragma unroll 1
     for (uint32_t e = (uint32_t)lane; e < n; e += 32) {
         const uint2 pr = xl[e];
         const int bin = exact_bin(prm, T, m.us, m.n_total, pr.x, pr.y);
-        cnt++;
         if (bin >= 0) {
             const uint32_t k = (uint32_t)bin / (uint32_t)prm.n_mu, j = (uint32_t)bin % (uint32_t)prm.n_mu;
             const uint32_t col = MU ? j + (uint32_t)dp.CO : 0u;
@@ -542,7 +582,6 @@ __device__ __forceinline__ uint32_t recheck(const CountParams &prm, const Direct
         }
     }
     __syncwarp();
-    return cnt;
 }
 
 // this lane's b-points of the tile (buffer slots 32 p + lane, packed in
@@ -580,9 +619,9 @@ __device__ __forceinline__ void load_tile(const float4 *buf, uint32_t nb, int la
 // add is taken back and the pair joins the recheck list.
 template <int V, int R, int LOGC, bool CHK>
 __device__ __forceinline__ void tile(const CountParams &prm, const DirectParams &dp, const Mesh &m,
-                                     const unsigned long long *T, const WarpMem &wm, const Addr &ad, uint32_t nb,
-                                     uint32_t nself, uint32_t na, uint32_t a0, int lane, uint32_t &n_list,
-                                     unsigned long long &n_exact, unsigned long long &n_cand)
+                                     const unsigned long long *T, const WarpMem &wm,
+                                     const Addr<(V > 0), R, LOGC> &ad, uint32_t nb, uint32_t nself, uint32_t na,
+                                     uint32_t a0, int lane, uint32_t &n_list)
 {
     constexpr bool MU = V > 0, MID = V == 2;
     float2 BX[NQ], BY[NQ], BZ[NQ];
@@ -601,7 +640,7 @@ __device__ __forceinline__ void tile(const CountParams &prm, const DirectParams 
     uint32_t live = 0;
 #pragma unroll
     for (int p = 0; p < NP; p++) live |= (32u * (uint32_t)p + (uint32_t)lane < nb ? 1u : 0u) << p;
-    n_cand += (unsigned long long)nb * na;
+    if (lane == 0) wm.st->n_cand += (unsigned long long)nb * na;
     constexpr int LS = Sh<R, LOGC>::LS, LT = Sh<R, LOGC>::LT;
     const K2 k2{u64of(make_float2(dp.tiny, dp.tiny)), u64of(make_float2(MAG_S, MAG_S)), u64of(make_float2(-1.0f, -1.0f)),
                 u64of(make_float2(MAG_S - 0.5f, MAG_S - 0.5f)), u64of(make_float2(MAG_T, MAG_T)),
@@ -640,18 +679,19 @@ __device__ __forceinline__ void tile(const CountParams &prm, const DirectParams 
                 }
                 n_list += __popc(mk);
                 if (n_list >= XCAP - 32) {
-                    n_exact += recheck<MU, R, LOGC>(prm, dp, m, T, wm.xl, n_list, ad.hb, lane);
+                    recheck<MU, R, LOGC>(prm, dp, m, T, wm, n_list, ad.hb(dp), lane);
                     n_list = 0;
                 }
             }
         }
     };
+    const uint32_t dump = CHK ? ad.dump(prm, dp) : 0u;
     uint32_t ai = 0;
 #pragma unroll 1
     for (; ai + 1 < na; ai += 2) {
         const ARec a = load_a<MID>(wm.arec, ai), a2 = load_a<MID>(wm.arec, ai + 1);
-        const bool u0 = apoint<V, CHK, LS, LT>(BX, BY, BZ, a, k2, dp.cs, dp.s_top, ad.Kl, a0 + ai, IB, ad.dump);
-        const bool u1 = apoint<V, CHK, LS, LT>(BX, BY, BZ, a2, k2, dp.cs, dp.s_top, ad.Kl, a0 + ai + 1, IB, ad.dump);
+        const bool u0 = apoint<V, CHK, LS, LT>(BX, BY, BZ, a, k2, dp.cs, dp.s_top, ad.Kl, a0 + ai, IB, dump);
+        const bool u1 = apoint<V, CHK, LS, LT>(BX, BY, BZ, a2, k2, dp.cs, dp.s_top, ad.Kl, a0 + ai + 1, IB, dump);
         if (__any_sync(0xffffffffu, u0 || u1)) {
 #pragma unroll 1
             for (uint32_t j = ai; j < ai + 2; j++) settle(j);
@@ -660,7 +700,7 @@ __device__ __forceinline__ void tile(const CountParams &prm, const DirectParams 
     if (ai < na) {   // the last a-point of an odd chunk
         const ARec a = load_a<MID>(wm.arec, ai);
         if (__any_sync(0xffffffffu,
-                       apoint<V, CHK, LS, LT>(BX, BY, BZ, a, k2, dp.cs, dp.s_top, ad.Kl, a0 + ai, IB, ad.dump)))
+                       apoint<V, CHK, LS, LT>(BX, BY, BZ, a, k2, dp.cs, dp.s_top, ad.Kl, a0 + ai, IB, dump)))
             settle(ai);
     }
     __syncwarp();
@@ -675,15 +715,17 @@ __device__ __forceinline__ float4 bpoint(const DirectParams &dp, uint32_t i, uin
                        __fmul_rn(__int2float_rn((int)(uz - oz)), dp.inv_qds), __uint_as_float(i));
 }
 
-// The unit: a-chunk [un.a0, un.a1) of cell un.cell against the term's neighbourhood.
+// The unit: a-chunk [un.a0, un.a1) of the cells un.cell .. (dp.G cells along x, fewer at the row's end) against the
+// term's neighbourhood.
 template <int V, int R, int LOGC>
 __device__ __forceinline__ void unit(const CountParams &prm, const DirectParams &dp, const Mesh &m,
-                                     const unsigned long long *T, const WarpMem &wm, const Addr &ad, const Unit &un,
-                                     const Term &tm, int lane, uint32_t &n_list, unsigned long long &n_exact,
-                                     unsigned long long &n_cand)
+                                     const unsigned long long *T, const WarpMem &wm,
+                                     const Addr<(V > 0), R, LOGC> &ad, const Unit &un, const Term &tm, int lane,
+                                     uint32_t &n_list)
 {
     const int n_c = prm.n_c;
     const int ax = un.cell % n_c, ay = (un.cell / n_c) % n_c, az = un.cell / (n_c * n_c);
+    const int ax1 = min(ax + dp.G, n_c) - 1;   // the last cell
     const uint32_t ox = m.orig[ax], oy = m.orig[ay], oz = m.orig[az];
     const size_t N = m.n_total;
     const uint32_t a0 = un.a0, na = un.a1 - un.a0;
@@ -698,6 +740,7 @@ __device__ __forceinline__ void unit(const CountParams &prm, const DirectParams 
         o2z = 2.0f * __fmul_rn(__ll2float_rn(prm.obs[2] - (long long)oz), dp.inv_qds);
     }
     float lx = INFINITY, ly = INFINITY, lz = INFINITY, hx = -INFINITY, hy = -INFINITY, hz = -INFINITY;
+#pragma unroll 1
     for (uint32_t i = (uint32_t)lane; i < na; i += 32) {
         const size_t g = a0 + i;
         const float4 p = bpoint(dp, (uint32_t)g, m.us[g], m.us[N + g], m.us[2 * N + g], ox, oy, oz);
@@ -741,6 +784,7 @@ __device__ __forceinline__ void unit(const CountParams &prm, const DirectParams 
     const bool periodic = prm.geometry == TPCF_PERIODIC;
     const uint32_t *cs = m.cellstart + (size_t)tm.cat_b * prm.n_cells;
     uint32_t n_run = 0, total = 0, self0 = 0, self1 = 0;
+#pragma unroll 1
     for (int r0 = 0; r0 < prm.n_rows; r0 += 32) {
         const int r = r0 + lane;
         uint32_t s0[2], s1[2];
@@ -757,7 +801,7 @@ __device__ __forceinline__ void unit(const CountParams &prm, const DirectParams 
             }
             if (use) {
                 const uint32_t rowkey = ((uint32_t)z * n_c + (uint32_t)y) * n_c;
-                int xlo = ax - kx, xhi = ax + kx;
+                int xlo = ax - kx, xhi = ax1 + kx;
                 auto add = [&](uint32_t a, uint32_t b) {
                     if (b > a) {
                         s0[nl] = a;
@@ -767,8 +811,8 @@ __device__ __forceinline__ void unit(const CountParams &prm, const DirectParams 
                 };
                 if (tm.auto_pairs && dz == 0 && dy == 0) {
                     self0 = cs[rowkey + ax];
-                    self1 = cs[rowkey + ax + 1];
-                    xlo = ax + 1;
+                    self1 = cs[rowkey + ax1 + 1];
+                    xlo = ax1 + 1;
                 }
                 if (xlo <= xhi) {
                     if (periodic) {
@@ -790,10 +834,12 @@ __device__ __forceinline__ void unit(const CountParams &prm, const DirectParams 
             }
         }
         uint32_t pl = 0;
+#pragma unroll 1
         for (int i = 0; i < nl; i++) pl += s1[i] - s0[i];
         uint32_t n_all, p_all;
         const uint32_t n_ex = warp_exclusive_sum((uint32_t)nl, lane, n_all);
         uint32_t p_ex = warp_exclusive_sum(pl, lane, p_all);
+#pragma unroll 1
         for (int i = 0; i < nl; i++) {
             wm.runs[n_run + n_ex + i] = make_uint2(s0[i], total + p_ex);
             p_ex += s1[i] - s0[i];
@@ -815,10 +861,12 @@ __device__ __forceinline__ void unit(const CountParams &prm, const DirectParams 
     // call site per kind of tile keeps the kernel's hot code small.
     uint32_t nbuf = 0, cself = self0, c = 0;
     int g = 0;
+#pragma unroll 1
     for (;;) {
         uint32_t nself = 0;
         if (cself < self1) {   // the buffer is empty here: self points come first
             nself = min((uint32_t)TB, self1 - cself);
+#pragma unroll 1
             for (uint32_t e2 = (uint32_t)lane; e2 < nself; e2 += 32) {
                 const size_t gi = cself + e2;
                 wm.buf[e2] = bpoint(dp, (uint32_t)gi, m.us[gi], m.us[N + gi], m.us[2 * N + gi], ox, oy, oz);
@@ -826,6 +874,7 @@ __device__ __forceinline__ void unit(const CountParams &prm, const DirectParams 
             cself += nself;
             nbuf = nself;
         }
+#pragma unroll 1
         while (nbuf < TB && c < total) {
             uint32_t idx[4];
             bool ok[4];
@@ -833,6 +882,7 @@ __device__ __forceinline__ void unit(const CountParams &prm, const DirectParams 
             for (int k = 0; k < 4; k++) {
                 const uint32_t o2 = c + 32u * (uint32_t)k + (uint32_t)lane;
                 ok[k] = o2 < total;
+#pragma unroll 1
                 while (g + 1 < (int)n_run && wm.runs[g + 1].y <= o2) g++;
                 idx[k] = ok[k] ? wm.runs[g].x + (o2 - wm.runs[g].y) : 0u;
             }
@@ -860,9 +910,9 @@ __device__ __forceinline__ void unit(const CountParams &prm, const DirectParams 
         const uint32_t nt = min(nbuf, (uint32_t)TB);
         __syncwarp();
         if (nself)
-            tile<V, R, LOGC, true>(prm, dp, m, T, wm, ad, nt, nself, na, a0, lane, n_list, n_exact, n_cand);
+            tile<V, R, LOGC, true>(prm, dp, m, T, wm, ad, nt, nself, na, a0, lane, n_list);
         else
-            tile<V, R, LOGC, false>(prm, dp, m, T, wm, ad, nt, 0u, na, a0, lane, n_list, n_exact, n_cand);
+            tile<V, R, LOGC, false>(prm, dp, m, T, wm, ad, nt, 0u, na, a0, lane, n_list);
         // the leftovers (fewer than 128) move to the front
         const uint32_t left = nbuf - nt;
         if (left) {
@@ -884,16 +934,17 @@ __device__ __forceinline__ void unit(const CountParams &prm, const DirectParams 
     }
 }
 
-// drain the table into term t's int64 histogram and clear it (whole block)
+// one warp drains a table into term t's int64 histogram and clears it
 template <bool MU, int R, int LOGC>
 __device__ __forceinline__ unsigned long long drain(const CountParams &prm, const DirectParams &dp,
-                                                    const Term *terms, uint32_t *hist, uint32_t hwords, int t)
+                                                    const Term *terms, uint32_t *hist, uint32_t hwords, int t,
+                                                    int lane)
 {
-    __syncthreads();
     long long *const th = terms[t].hist;
     const int n_mu = prm.n_mu;
     unsigned long long binned = 0;
-    for (int b = threadIdx.x; b < prm.nbin; b += blockDim.x) {
+#pragma unroll 1
+    for (int b = lane; b < prm.nbin; b += 32) {
         const int k = b / n_mu, j = b % n_mu;
         unsigned long long sum = 0;
         // mu bin j: signed columns j and -1 - j
@@ -915,142 +966,236 @@ __device__ __forceinline__ unsigned long long drain(const CountParams &prm, cons
         if (sum) atomicAdd((unsigned long long *)&th[b], sum);
         binned += sum;
     }
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < hwords; i += blockDim.x) hist[i] = 0u;
-    __syncthreads();
+    __syncwarp();
+#pragma unroll 1
+    for (uint32_t i = (uint32_t)lane; i < hwords / 4; i += 32) ((uint4 *)hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
     return binned;
+}
+
+// The schedule's lock, taken by one lane of a warp.  The wait is bounded: it
+// can only run out if a warp of this block stopped running.
+__device__ __forceinline__ bool sched_lock(Sched &q)
+{
+#pragma unroll 1
+    for (unsigned i = 0; i < (1u << 24); i++) {
+        if (atomicCAS(&q.lock, 0u, 1u) == 0u) {
+            __threadfence_block();
+            return true;
+        }
+        __nanosleep(20);
+    }
+    return false;
+}
+__device__ __forceinline__ void sched_unlock(Sched &q)
+{
+    __threadfence_block();
+    atomicExch(&q.lock, 0u);
+}
+
+constexpr unsigned NO_UNIT = 0xFFFFFFFFu;
+
+// The block's claim is used up: one lane takes the next unit of the claim
+// that another warp made meanwhile, or makes a new one.  Claims shrink toward
+// the end (guided self-scheduling): a block takes half of the remaining units'
+// fair share, at most csize units and at least csize / 32 or one per warp, so
+// the last claims, which set the launch's tail, are short.  A stale read of
+// the counter only changes a claim's length; the atomic add keeps the claims
+// disjoint and covering.
+__device__ __forceinline__ unsigned claim_more(Sched &q, unsigned *claim, uint32_t u_lo, uint32_t span, uint32_t csize,
+                                            int *status)
+{
+    unsigned u = NO_UNIT;
+    if (!sched_lock(q)) {
+        atomicOr(status, STATUS_TIMEOUT);
+        return u;
+    }
+    const unsigned long long c = atomicAdd(&q.claim, 1ull);
+    if ((uint32_t)c < (uint32_t)(c >> 32)) {
+        u = (uint32_t)c;
+    } else {
+        const uint32_t g = *(volatile unsigned *)claim;
+        const uint32_t rem = g < span ? span - g : 0u;
+        const uint32_t cmin = min(csize, max(csize / 32u, (uint32_t)DIRECT_WARPS));
+        const uint32_t sz = max(cmin, min(csize, rem / (2u * gridDim.x)));
+        const uint32_t c0 = rem ? atomicAdd(claim, sz) : span;
+        if (c0 < span) {
+            u = u_lo + c0;
+            atomicExch(&q.claim,
+                       (unsigned long long)(u + 1u) | (unsigned long long)(u_lo + min(span, c0 + sz)) << 32);
+        }
+    }
+    sched_unlock(q);
+    return u;
+}
+
+// units a table may take between two drains: a unit adds at most
+// unit_pair_bound to any of its 32-bit counters
+__device__ __forceinline__ unsigned most_units(const DirectParams &dp)
+{
+    return (unsigned)min(0x7fffffffull, ((1ull << 32) - 1ull) / dp.unit_pair_bound);
+}
+
+// The warp (all lanes) leaves its table, if it has one, draining it when it is
+// the last to leave, and, if u is a unit, enters the table of u's term: the one
+// that counts it, or a free one (a bounded wait for a drain).  Returns the
+// table, -1 when there is none (NO_UNIT, or the wait ran out).  n_list pairs
+// still await their exact recheck in the table that is left, whose base for
+// this lane is hb.
+template <bool MU, int R, int LOGC>
+__device__ __forceinline__ int switch_table(const CountParams &prm, const DirectParams &dp, const Mesh &m,
+                                         const Term *terms, const Unit *units, const uint32_t *ustart,
+                                         const unsigned long long *T, const WarpMem &wm, Sched &q,
+                                         unsigned char *tables, uint32_t hstride, uint32_t hb, unsigned u,
+                                         uint32_t n_list, int *status)
+{
+    const int lane = threadIdx.x & 31, tab = wm.st->tab;
+    if (tab >= 0) {
+        if (n_list) recheck<MU, R, LOGC>(prm, dp, m, T, wm, n_list, hb, lane);
+        __syncwarp();
+        unsigned last = 0;
+        if (lane == 0 && sched_lock(q)) {
+            last = --q.ref[tab] == 0u;
+            if (last) q.term[tab] = DRAINING;
+            sched_unlock(q);
+        }
+        if (__shfl_sync(0xffffffffu, last, 0)) {
+            unsigned long long bn = drain<MU, R, LOGC>(prm, dp, terms, (uint32_t *)(tables + (size_t)tab * hstride),
+                                                       hstride / 4u, wm.st->term, lane);
+#pragma unroll
+            for (int s2 = 16; s2 > 0; s2 >>= 1) bn += __shfl_down_sync(0xffffffffu, bn, s2);
+            if (lane == 0) {
+                wm.st->binned += bn;
+                if (sched_lock(q)) {
+                    q.term[tab] = FREE;
+                    sched_unlock(q);
+                }
+            }
+        }
+    }
+    int k = -1;
+    if (u != NO_UNIT && lane == 0) {
+        const int t = units[u].term;
+        const uint32_t t_lo = ustart[(size_t)t * dp.n_groups], t_hi = ustart[(size_t)(t + 1) * dp.n_groups];
+        const unsigned most = most_units(dp);
+#pragma unroll 1
+        for (unsigned i = 0; i < (1u << 24) && k < 0; i++) {
+            if (!sched_lock(q)) break;
+#pragma unroll 1
+            for (int j = 0; j < dp.NT; j++)
+                if (q.term[j] == t && atomicAdd(&q.n_used[j], 1u) < most) k = j;
+            if (k >= 0) {
+                q.ref[k]++;
+            } else {
+#pragma unroll 1
+                for (int j = 0; j < dp.NT; j++)
+                    if (k < 0 && q.term[j] == FREE) k = j;
+                if (k >= 0) {
+                    q.term[k] = t;
+                    q.ref[k] = 1u;
+                    atomicExch(&q.n_used[k], 1u);
+                }
+            }
+            sched_unlock(q);
+            if (k < 0) __nanosleep(200);
+        }
+        if (k < 0) atomicOr(status, STATUS_TIMEOUT);
+        wm.st->tab = k;
+        wm.st->term = t;
+        wm.st->t_lo = t_lo;
+        wm.st->t_hi = t_hi;
+    }
+    return __shfl_sync(0xffffffffu, k, 0);
 }
 
 template <int V, int R, int W, int LOGC>
 __global__ void __launch_bounds__(W * 32, 1)
     pairdirect_kernel(const __grid_constant__ CountParams prm, const __grid_constant__ DirectParams dp, const Mesh m,
                       const Term *__restrict__ terms, const Unit *__restrict__ units,
-                      const uint32_t *__restrict__ n_units_p, unsigned *__restrict__ claim,
-                      unsigned long long *__restrict__ stats, int term_only, int chunk)
+                      const uint32_t *__restrict__ ustart, const uint32_t *__restrict__ n_units_p,
+                      unsigned *__restrict__ claim, unsigned long long *__restrict__ stats, int *__restrict__ status,
+                      int term_only, int chunk)
 {
     constexpr bool MU = V > 0;
-    const DOff o = d_off(prm.n_s, prm.n_rows, R, dp.C, W);
+    const DOff o = d_off(prm.n_s, prm.n_rows, R, dp.C, dp.NT, W);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const unsigned long long t_start = gtimer();
-    uint32_t *hist = (uint32_t *)(dsm + o.hist);
     unsigned long long *Tsh = (unsigned long long *)(dsm + o.T);
-    unsigned *misc = (unsigned *)(dsm + o.misc);
-    const uint32_t hwords = (uint32_t)(dp.rows * dp.C * R);
-    for (uint32_t i = tid; i < hwords; i += blockDim.x) hist[i] = 0u;
+    Sched &q = *(Sched *)(dsm + o.misc);
+    const uint32_t hwords = o.hstride / 4u;
+#pragma unroll 1
+    for (uint32_t i = tid; i < hwords * (uint32_t)dp.NT; i += blockDim.x) ((uint32_t *)(dsm + o.hist))[i] = 0u;
+#pragma unroll 1
     for (int i = tid; i <= prm.n_s; i += blockDim.x) Tsh[i] = prm.T[i];
+    if (tid == 0) {
+        q.claim = 0ull;
+        q.lock = 0u;
+        for (int k = 0; k < MAX_NT; k++) {
+            q.term[k] = FREE;
+            q.ref[k] = q.n_used[k] = 0u;
+        }
+    }
 
     unsigned char *wr = dsm + o.warp0 + (size_t)warp * o.wstride;
-    const WarpMem wm{(float4 *)(wr + o.arec), (float4 *)(wr + o.buf), (uint2 *)(wr + o.runs), (uint2 *)(wr + o.xl)};
-    Addr ad;
-    ad.hb = saddr(dsm) + o.hist + 4u * ((uint32_t)lane & (uint32_t)(R - 1));
-    constexpr int LS = Sh<R, LOGC>::LS, LT = Sh<R, LOGC>::LT;
-    if (MU)
-        ad.Kl = ad.hb + ((uint32_t)dp.CO << LT) - (MAG_S_BITS << LS) - (MAG_T_BITS << LT);
-    else
-        ad.Kl = ad.hb - (MAG_S_BITS << LS);
-    ad.dump = ad.hb + ((uint32_t)prm.n_s << LS);
+    const WarpMem wm{(float4 *)(wr + o.arec), (float4 *)(wr + o.buf), (uint2 *)(wr + o.runs), (uint2 *)(wr + o.xl),
+                     (WarpState *)(wr + o.st)};
+    if (lane == 0) *wm.st = WarpState{0ull, 0ull, 0ull, gtimer(), -1, -1, 0u, 0u};
     uint32_t n_list = 0;
-    unsigned long long n_exact = 0, n_cand = 0, binned = 0;
 
-    // Chunks of consecutive units are claimed by the block and worked through
-    // term by term, their units claimed one at a time by the warps.  The table
-    // is drained when the term changes, or before the pairs added since the
-    // last drain could reach 2^31 in one counter (a unit adds at most
-    // unit_pair_bound to any counter, and a chunk at most 2^30).  With
-    // term_only >= 0 (one launch per term) only that term's units are claimed.
+    // The block claims chunks of consecutive units and its warps take them one
+    // at a time, each on its own: no barrier separates claims or terms.  A
+    // table counts one term.  A warp whose next unit belongs to another term
+    // (or whose table could wrap) leaves its table and enters the one of that
+    // term or a free one; the last warp to leave a table drains it.  With two
+    // tables or more the warps of a block pass from one term to the next
+    // without waiting for each other (one table is taken only where two do not
+    // fit: 19.9 ms instead of 15.6 on eight mocks of 100 000 points).  With a
+    // block barrier after every claim and before every drain, each of them
+    // waiting for the block's slowest warp (a unit takes 0.05 to 0.3 ms), the
+    // barriers cost 18 % of the warps' time on two such mocks: kernel times 16.4
+    // -> 15.6 ms for eight, 60.7 -> 59.6 for three of a million points, 3.88 ->
+    // 3.61 for eight of 60 000; 32.7 -> 32.8 on cut-sky mocks, whose terms are long
+    // and units short.  Units of a few points (four per cell) suffer, since
+    // warps at different places of the code share less of the instruction
+    // cache (0.32 -> 0.42 ms on 16 mocks of 4000 points); the tuner takes larger
+    // cells there (0.24 ms).  With term_only >= 0 (one launch per term) only
+    // that term's units are claimed.
     const uint32_t n_all = *n_units_p;
     uint32_t u_lo = 0, u_hi = n_all;
     if (term_only >= 0) {
-        uint32_t lo = 0, hi = n_all;   // first unit of a term >= term_only
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (units[mid].term < term_only) lo = mid + 1; else hi = mid;
-        }
-        u_lo = lo;
-        hi = n_all;                    // first unit of a term > term_only
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (units[mid].term <= term_only) lo = mid + 1; else hi = mid;
-        }
-        u_hi = lo;
+        u_lo = ustart[(size_t)term_only * dp.n_groups];
+        u_hi = ustart[(size_t)(term_only + 1) * dp.n_groups];
     }
-    // Claims shrink toward the end (guided self-scheduling): a block takes
-    // half of the remaining units' fair share, at most chunk units and at
-    // least chunk / 32 or two per warp (fewer would leave warps idle), so the
-    // last claims, which set the launch's tail, are short.  A stale read of
-    // the counter only changes a claim's length; the atomic add keeps the
-    // claims disjoint and covering.
-    const uint32_t csize = (uint32_t)chunk, span = u_hi - u_lo;
-    const uint32_t cmin = min(csize, max(csize / 32u, 2u * (uint32_t)W));
-    int cur_term = -1;
-    unsigned long long since = 0;
+    const uint32_t span = u_hi - u_lo;
+    const unsigned most = most_units(dp);
+    Addr<MU, R, LOGC> ad{0u};
     __syncthreads();
+#pragma unroll 1
     for (;;) {
-        if (tid == 0) {
-            const uint32_t cur = *(volatile unsigned *)claim;
-            const uint32_t rem = cur < span ? span - cur : 0u;
-            const uint32_t sz = max(cmin, min(csize, rem / (2u * gridDim.x)));
-            misc[0] = u_lo + atomicAdd(claim, sz);
-            misc[2] = sz;
+        // the next unit; `stay`: it goes to the warp's own table
+        unsigned u = NO_UNIT, stay = 0;
+        if (lane == 0) {
+            const unsigned long long c = atomicAdd(&q.claim, 1ull);
+            if ((uint32_t)c < (uint32_t)(c >> 32)) u = (uint32_t)c;
+            else u = claim_more(q, claim, u_lo, span, (uint32_t)chunk, status);
+            stay = u >= wm.st->t_lo && u < wm.st->t_hi && atomicAdd(&q.n_used[wm.st->tab], 1u) < most;
         }
-        __syncthreads();
-        const uint32_t c0 = misc[0];
-        if (c0 >= u_hi) break;
-        const uint32_t c1 = min(u_hi, c0 + misc[2]);
-        uint32_t s = c0;
-        while (s < c1) {
-            const int t = units[s].term;
-            // the end of term t inside [s, c1)
-            uint32_t lo = s, hi = c1;
-            while (hi - lo > 1) {
-                const uint32_t mid = (lo + hi) >> 1;
-                if (units[mid].term == t) lo = mid; else hi = mid;
-            }
-            const uint32_t e = hi;
-            const unsigned long long seg = (unsigned long long)(e - s) * dp.unit_pair_bound;
-            if (cur_term >= 0 && (t != cur_term || since + seg >= (1ull << 31))) {
-                if (n_list) {   // pending rechecks belong to the table being drained
-                    n_exact += recheck<MU, R, LOGC>(prm, dp, m, Tsh, wm.xl, n_list, ad.hb, lane);
-                    n_list = 0;
-                }
-                binned += drain<MU, R, LOGC>(prm, dp, terms, hist, hwords, cur_term);
-                since = 0;
-            }
-            cur_term = t;
-            since += seg;
-            if (tid == 0) misc[1] = s;
-            __syncthreads();
-            const Term tm = terms[t];
-            for (;;) {
-                uint32_t u = 0;
-                if (lane == 0) u = atomicAdd(&misc[1], 1u);
-                u = __shfl_sync(0xffffffffu, u, 0);
-                if (u >= e) break;
-                unit<V, R, LOGC>(prm, dp, m, Tsh, wm, ad, units[u], tm, lane, n_list, n_exact, n_cand);
-            }
-            __syncthreads();
-            s = e;
-        }
-    }
-    if (cur_term >= 0) {
-        if (n_list) {
-            n_exact += recheck<MU, R, LOGC>(prm, dp, m, Tsh, wm.xl, n_list, ad.hb, lane);
+        u = __shfl_sync(0xffffffffu, u, 0);
+        if (!__shfl_sync(0xffffffffu, stay, 0)) {
+            const int k = switch_table<MU, R, LOGC>(prm, dp, m, terms, units, ustart, Tsh, wm, q, dsm + o.hist,
+                                                    o.hstride, ad.hb(dp), u, n_list, status);
             n_list = 0;
+            if (k < 0) break;
+            ad.Kl = saddr(dsm) + o.hist + (uint32_t)k * o.hstride + 4u * ((uint32_t)lane & (uint32_t)(R - 1)) +
+                    Addr<MU, R, LOGC>::shift(dp);
         }
-        binned += drain<MU, R, LOGC>(prm, dp, terms, hist, hwords, cur_term);
-    }
-    unsigned long long ex = n_exact, bn = binned, cd = lane == 0 ? n_cand : 0ull;
-#pragma unroll
-    for (int s2 = 16; s2 > 0; s2 >>= 1) {
-        ex += __shfl_down_sync(0xffffffffu, ex, s2);
-        bn += __shfl_down_sync(0xffffffffu, bn, s2);
-        cd += __shfl_down_sync(0xffffffffu, cd, s2);
+        const Unit un = units[u];
+        unit<V, R, LOGC>(prm, dp, m, Tsh, wm, ad, un, terms[un.term], lane, n_list);
     }
     if (lane == 0) {
-        atomicAdd(&stats[0], cd);
-        atomicAdd(&stats[1], bn);
-        atomicAdd(&stats[2], ex);
-        record_warp_span(stats, t_start);
+        atomicAdd(&stats[0], wm.st->n_cand);
+        atomicAdd(&stats[1], wm.st->binned);
+        atomicAdd(&stats[2], wm.st->n_exact);
+        record_warp_span(stats, wm.st->t_start);
     }
 }
 
@@ -1066,11 +1211,13 @@ void *select_direct(int V, int R, int W, int logC)
 {
     if (W != DIRECT_WARPS) return nullptr;
     constexpr int DW = DIRECT_WARPS;
-    if (V == 0) return R == 32 ? dkernel<0, 32, DW, 0>() : dkernel<0, 16, DW, 0>();
-    if (V == 1 && logC == 5) return R == 32 ? dkernel<1, 32, DW, 5>() : dkernel<1, 16, DW, 5>();
-    if (V == 1 && logC == 6) return R == 32 ? dkernel<1, 32, DW, 6>() : dkernel<1, 16, DW, 6>();
-    if (V == 2 && logC == 5) return R == 32 ? dkernel<2, 32, DW, 5>() : dkernel<2, 16, DW, 5>();
-    if (V == 2 && logC == 6) return R == 32 ? dkernel<2, 32, DW, 6>() : dkernel<2, 16, DW, 6>();
+    if (V == 0) return R == 32 ? dkernel<0, 32, DW, 0>() : nullptr;
+    if (V == 1 && logC == 4) return R == 32 ? dkernel<1, 32, DW, 4>() : (R == 16 ? dkernel<1, 16, DW, 4>() : nullptr);
+    if (V == 2 && logC == 4) return R == 32 ? dkernel<2, 32, DW, 4>() : (R == 16 ? dkernel<2, 16, DW, 4>() : nullptr);
+    if (V == 1 && logC == 5) return R == 32 ? dkernel<1, 32, DW, 5>() : (R == 16 ? dkernel<1, 16, DW, 5>() : dkernel<1, 8, DW, 5>());
+    if (V == 1 && logC == 6) return R == 16 ? dkernel<1, 16, DW, 6>() : (R == 8 ? dkernel<1, 8, DW, 6>() : nullptr);
+    if (V == 2 && logC == 5) return R == 32 ? dkernel<2, 32, DW, 5>() : (R == 16 ? dkernel<2, 16, DW, 5>() : dkernel<2, 8, DW, 5>());
+    if (V == 2 && logC == 6) return R == 16 ? dkernel<2, 16, DW, 6>() : (R == 8 ? dkernel<2, 8, DW, 6>() : nullptr);
     return nullptr;
 }
 
@@ -1078,9 +1225,9 @@ int mode_of(const DirectParams &d, bool mu) { return !mu ? 0 : (d.mid ? 2 : 1); 
 
 }  // namespace
 
-size_t pairdirect_smem_bytes(const CountParams &p, int R, int C, int W)
+size_t pairdirect_smem_bytes(const CountParams &p, int R, int C, int NT, int W)
 {
-    return d_off(p.n_s, p.n_rows, R, C, W).end;
+    return d_off(p.n_s, p.n_rows, R, C, NT, W).end;
 }
 
 cudaError_t pairdirect_set_attrs(const DirectParams &d, int mu)
@@ -1102,14 +1249,14 @@ int pairdirect_max_blocks_per_sm(const DirectParams &d, int mu)
 }
 
 cudaError_t launch_pairdirect(const CountParams &p, const DirectParams &d, const Mesh &m, const Term *terms,
-                              const Unit *units, const uint32_t *n_units, unsigned *claim, unsigned long long *stats,
-                              const PairLaunch &pl, cudaStream_t s)
+                              const Unit *units, const uint32_t *ustart, const uint32_t *n_units, unsigned *claim,
+                              unsigned long long *stats, int *status, const PairLaunch &pl, cudaStream_t s)
 {
     void *k = select_direct(mode_of(d, p.n_mu > 1), d.R, d.W, d.logC);
     if (!k) return cudaErrorInvalidValue;
     const int term_only = pl.persistent ? -1 : pl.term;
-    void *args[] = {(void *)&p,      (void *)&d,     (void *)&m,     (void *)&terms,     (void *)&units,
-                    (void *)&n_units, (void *)&claim, (void *)&stats, (void *)&term_only, (void *)&pl.chunk};
+    void *args[] = {(void *)&p,       (void *)&d,     (void *)&m,     (void *)&terms,  (void *)&units,     (void *)&ustart,
+                    (void *)&n_units, (void *)&claim, (void *)&stats, (void *)&status, (void *)&term_only, (void *)&pl.chunk};
     return cudaLaunchKernel(k, dim3(pl.blocks), dim3(d.W * 32), args, (size_t)d.smem, s);
 }
 

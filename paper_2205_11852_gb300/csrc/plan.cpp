@@ -392,7 +392,7 @@ int build_plan(const tpcf_binning &b, int subdiv, unsigned long long max_cells, 
 // 1.1 (n_mu 2E + 1.5 ulp(n_mu Xb + 1) + n_mu rho (n_s + 1) + n_mu dsq) (the
 // common scale cancels in mu) plus the bias of the d2 addend (see below).
 bool build_direct(const tpcf_binning &b, const Plan &pl, int smem_sm, int smem_block, int reserved,
-                  unsigned long long max_cat, DirectParams &d)
+                  unsigned long long max_cat, int group, DirectParams &d)
 {
     const CountParams &p = pl.prm;
     std::memset(&d, 0, sizeof(d));
@@ -407,7 +407,17 @@ bool build_direct(const tpcf_binning &b, const Plan &pl, int smem_sm, int smem_b
     const double u24 = std::ldexp(1.0, -24);
     const double kappa = std::fabs((double)inv * qds - 1.0);
     const double Wmax = std::ldexp(1.0, p.bits) / (double)p.n_c + 1.0;
-    const double Xg = (double)(pl.K + 1) * Wmax;
+    // a unit spans `group` cells along x, its neighbourhood K more on either
+    // side: in a periodic box every neighbour within the last edge must lie
+    // within half a box of the unit's corner (coordinates are differences from
+    // it, modulo the box), and no cell may be a neighbour from both sides
+    if (group > 1 && b.geometry == TPCF_PERIODIC) {
+        const double smax_q = std::sqrt((double)p.T[b.n_s]) + 2.0;
+        if (!(group * Wmax + smax_q < std::ldexp(1.0, 31)) || group + 2 * pl.K > p.n_c) return false;
+    }
+    d.G = group;
+    d.n_groups = p.n_c * p.n_c * ((p.n_c + group - 1) / group);
+    const double Xg = (double)(pl.K + group) * Wmax;
     const double Xb = Xg / qds * (1.0 + std::ldexp(1.0, -20));
     const double E = 0.5 * ulp_f32(Xg) / qds * (1.0 + std::ldexp(1.0, -20)) + 0.5 * ulp_f32(Xb);
     const double n_s = p.n_s, n_mu = p.n_mu;
@@ -467,7 +477,7 @@ bool build_direct(const tpcf_binning &b, const Plan &pl, int smem_sm, int smem_b
         d.mid = mid ? 1 : 0;
         int lc = 0;
         while ((1 << lc) < 2 * d.CO) lc++;
-        if (lc < 5) lc = 5;
+        if (lc < 4) lc = 4;
         if (lc > 6) return false;
         d.logC = lc;
     }
@@ -482,24 +492,29 @@ bool build_direct(const tpcf_binning &b, const Plan &pl, int smem_sm, int smem_b
     d.C = 1 << d.logC;
     d.rows = p.n_s + 1;
     // one block of DIRECT_WARPS warps per SM (their registers fill the
-    // register file), with 32 histogram copies when they fit beside the
-    // warps' regions, else 16
+    // register file).  At least two tables, so that its warps pass from term to
+    // term without waiting for each other, before copies (see pairdirect.cu);
+    // four where they cost little shared memory
     const long long budget = (long long)std::min(smem_block, smem_sm - reserved);
-    for (int W : {DIRECT_WARPS}) {
-        for (int R : {32, 16}) {
-            const long long need = (long long)pairdirect_smem_bytes(p, R, d.C, W);
-            if (need <= budget) {
-                d.R = R;
-                d.W = W;
-                d.smem = (int)need;
-                // in one unit a lane pairs at most 64 a-points with at most
-                // max_cat / 32 + 16 b-points (its tile slots), and 32 / R
-                // lanes share a counter copy
-                d.unit_pair_bound = (unsigned long long)DIRECT_ACHUNK *
-                                    (max_cat / (unsigned long long)R + 512ull / (unsigned long long)R + 16ull);
-                return true;
-            }
-        }
+    constexpr int W = DIRECT_WARPS;
+    static const struct {
+        int NT, R;
+    } opts[] = {{4, 32}, {2, 32}, {4, 16}, {2, 16}, {2, 8}, {1, 16}, {1, 8}};
+    for (const auto &op : opts) {
+        if (!mu && op.R != 32) continue;
+        if ((op.R == 32 && d.logC > 5) || (op.R == 8 && d.logC < 5)) continue;
+        const long long need = (long long)pairdirect_smem_bytes(p, op.R, d.C, op.NT, W);
+        if (need > budget) continue;
+        d.NT = op.NT;
+        d.R = op.R;
+        d.W = W;
+        d.smem = (int)need;
+        // in one unit a lane pairs at most 64 a-points with at most
+        // max_cat / 32 + 16 b-points (its tile slots), and 32 / R
+        // lanes share a counter copy
+        d.unit_pair_bound = (unsigned long long)DIRECT_ACHUNK * (max_cat / (unsigned long long)op.R +
+                                                                 512ull / (unsigned long long)op.R + 16ull);
+        return true;
     }
     return false;
 }

@@ -24,9 +24,10 @@ bool exact_threshold(double e, double L, int bits, unsigned long long &T);
 // binning does not suit it (s bins not linear from 0, a midpoint line of
 // sight with mu bins, a histogram beyond shared memory, FP32 bands too wide).
 // smem_sm / smem_block: the device's shared memory per SM and per block
-// (opt-in), reserved: the per-block reservation.
+// (opt-in), reserved: the per-block reservation.  group: cells along x that
+// share a unit; false when the periodic box is too small for it.
 bool build_direct(const tpcf_binning &b, const Plan &pl, int smem_sm, int smem_block, int reserved,
-                  unsigned long long max_cat, DirectParams &d);
+                  unsigned long long max_cat, int group, DirectParams &d);
 // max_cells caps the mesh (n_c^3); cells never shrink below s_max / subdiv.
 int build_plan(const tpcf_binning &b, int subdiv, unsigned long long max_cells, Plan &pl, std::string &err);
 

@@ -86,6 +86,7 @@ struct CountParams {
 // cell; the error bounds behind m, cs and d2min are derived in plan.cpp.
 struct DirectParams {
     int R;             // histogram copies (lane l adds to copy l mod R)
+    int NT;            // tables (terms) a block counts at a time, 1 to DIRECT_TABLES
     int W;             // warps per block (one block per SM)
     int C;             // histogram columns, 1 << logC: signed mu columns from -CO, or 1 (s only)
     int logC;
@@ -101,7 +102,8 @@ struct DirectParams {
     float tiny;        // d2 addend (keeps rsqrt finite; with mu bins it also bounds r)
     float hit;         // filter: squared box distance (bin^2) below which a b-point is kept
     float s_top;       // 2^23 + n_s: the clamped row of pairs beyond the last edge
-    float pad2;
+    int G;             // cells along x that share a unit
+    int n_groups;      // groups of cells per catalogue: n_c^2 ceil(n_c / G)
     // midpoint line of sight: t = n_mu mu is certain when |t - floor(t) - 1/2| <= c05 - c1 r - c3 rl
     // (r = 1 / |d|, rl = 1 / |l| as computed); tinyl keeps rl finite
     float c1, c3, c05, tinyl;
@@ -133,12 +135,12 @@ cudaError_t launch_scatter(const Cat *cats, int n_cat, uint32_t max_n, const Cou
                            const uint32_t *uq, const uint32_t *keys, const uint32_t *cellstart,
                            uint32_t *cursor, const uint32_t *orig, uint32_t n_total, uint32_t *us,
                            float4 *pf, uint16_t *pcx, cudaStream_t s);
-cudaError_t launch_unit_count(const Term *terms, int n_terms, const Cat *cats, int n_cells,
-                              const uint32_t *cellstart, int chunk, uint32_t *ucount, cudaStream_t s);
+// work units of groups of G consecutive cells along x (n_c cells per axis): ucount[n_terms * n_c^2 ceil(n_c / G)]
+cudaError_t launch_unit_count(const Term *terms, int n_terms, int n_c, int G, const uint32_t *cellstart, int chunk,
+                              uint32_t *ucount, cudaStream_t s);
 cudaError_t launch_stats_accum(const unsigned long long *stats, unsigned long long *acc, int first, cudaStream_t s);
-cudaError_t launch_unit_fill(const Term *terms, int n_terms, const Cat *cats, int n_cells,
-                             const uint32_t *cellstart, int chunk, const uint32_t *ustart, Unit *units,
-                             cudaStream_t s);
+cudaError_t launch_unit_fill(const Term *terms, int n_terms, int n_c, int G, const uint32_t *cellstart, int chunk,
+                             const uint32_t *ustart, Unit *units, cudaStream_t s);
 
 struct PairLaunch {
     int blocks;            // grid size
@@ -161,10 +163,11 @@ int paircount_max_blocks_per_sm(const CountParams &p, int warps_per_block, int s
 // direct pair counter (pairdirect.cu): one block of DIRECT_WARPS warps per SM, no global scratch
 constexpr int DIRECT_ACHUNK = 64;    // a-points per work unit
 constexpr int DIRECT_WARPS = 16;
+constexpr int DIRECT_TABLES = 4;     // histogram tables per block, at most
 cudaError_t launch_pairdirect(const CountParams &p, const DirectParams &d, const Mesh &m, const Term *terms,
-                              const Unit *units, const uint32_t *n_units, unsigned *claim, unsigned long long *stats,
-                              const PairLaunch &pl, cudaStream_t s);
-size_t pairdirect_smem_bytes(const CountParams &p, int R, int C, int W);
+                              const Unit *units, const uint32_t *ustart, const uint32_t *n_units, unsigned *claim,
+                              unsigned long long *stats, int *status, const PairLaunch &pl, cudaStream_t s);
+size_t pairdirect_smem_bytes(const CountParams &p, int R, int C, int NT, int W);
 cudaError_t pairdirect_set_attrs(const DirectParams &d, int mu);
 int pairdirect_max_blocks_per_sm(const DirectParams &d, int mu);
 
