@@ -379,12 +379,12 @@ __global__ void __launch_bounds__(32 * TS_WARPS)
 // that its norm lies in [1, 2): the number of sign changes is the number of
 // eigenvalues below x, without a division per step, and each step rounds like
 // the ratio form of the Sturm sequence, so the count is that of a matrix
-// within a few ulps of T.  t[i] = (d_i, e2_{i-1}), e2 at least 2^-120 (a
-// perturbation of T by 2^-60).  An exact zero becomes a tiny value of the
+// within a few ulps of T.  t[i] = (d_i, e2_{i-1}), e2 at least 2^-180 (a
+// perturbation of T by 2^-90).  An exact zero becomes a tiny value of the
 // opposite sign of p_{i-1}, which no later comparison can tell from it.  The
 // pair (p_i, p_{i-1}) is rescaled by a power of two (exactly) every four
-// steps: its larger member changes by 2^-123 to 2^3 per step, so nothing leaves
-// the normal range in between.  Returns the count; (m, ex): the last continuant
+// steps: its larger member changes by 2^-183 to 2^3 per step, so it stays
+// within 2^+-950 in between.  Returns the count; (m, ex): the last continuant
 // as m 2^ex.
 __device__ __forceinline__ int sturm_count(const double2 *t, int n, double x, double &m, int &ex)
 {
@@ -441,11 +441,17 @@ __global__ void __launch_bounds__(32) multisect_kernel(const double *__restrict_
     extern __shared__ double2 st[];   // [n]
     const int lane = threadIdx.x & 31, i = blockIdx.x;
     double lo = INFINITY, hi = -INFINITY, nrm = 0.0;
+    bool nan = false;
     for (int k = lane; k < n; k += 32) {
         const double r = (k > 0 ? fabs(e[k - 1]) : 0.0) + (k + 1 < n ? fabs(e[k]) : 0.0);
         lo = fmin(lo, d[k] - r);
         hi = fmax(hi, d[k] + r);
         nrm = fmax(nrm, fabs(d[k]) + r);
+        nan |= !(fabs(d[k]) + r < INFINITY);
+    }
+    if (__any_sync(0xffffffffu, nan)) {   // fmin and fmax pass over NaNs, and an infinite bracket does not close
+        if (lane == 0) w[i] = __longlong_as_double(0x7ff8000000000000ll);
+        return;
     }
     for (int o = 16; o > 0; o >>= 1) {
         lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
@@ -459,7 +465,7 @@ __global__ void __launch_bounds__(32) multisect_kernel(const double *__restrict_
     const int ks = ilogb(nrm);   // T / 2^ks has its norm in [1, 2)
     for (int k = lane; k < n; k += 32) {
         const double ek = k > 0 ? scalbn(e[k - 1], -ks) : 0.0;
-        st[k] = make_double2(scalbn(d[k], -ks), k > 0 ? fmax(ek * ek, 0x1p-120) : 0.0);
+        st[k] = make_double2(scalbn(d[k], -ks), k > 0 ? fmax(ek * ek, 0x1p-180) : 0.0);
     }
     __syncwarp();
     const double pad = 4e-16 * n;

@@ -1054,10 +1054,14 @@ __device__ __forceinline__ int switch_table(const CountParams &prm, const Direct
         if (n_list) recheck<MU, R, LOGC>(prm, dp, m, T, wm, n_list, hb, lane);
         __syncwarp();
         unsigned last = 0;
-        if (lane == 0 && sched_lock(q)) {
-            last = --q.ref[tab] == 0u;
-            if (last) q.term[tab] = DRAINING;
-            sched_unlock(q);
+        if (lane == 0) {
+            if (sched_lock(q)) {
+                last = --q.ref[tab] == 0u;
+                if (last) q.term[tab] = DRAINING;
+                sched_unlock(q);
+            } else {   // the table would never be drained
+                atomicOr(status, STATUS_TIMEOUT);
+            }
         }
         if (__shfl_sync(0xffffffffu, last, 0)) {
             unsigned long long bn = drain<MU, R, LOGC>(prm, dp, terms, (uint32_t *)(tables + (size_t)tab * hstride),
@@ -1069,6 +1073,8 @@ __device__ __forceinline__ int switch_table(const CountParams &prm, const Direct
                 if (sched_lock(q)) {
                     q.term[tab] = FREE;
                     sched_unlock(q);
+                } else {
+                    atomicOr(status, STATUS_TIMEOUT);
                 }
             }
         }
@@ -1078,12 +1084,16 @@ __device__ __forceinline__ int switch_table(const CountParams &prm, const Direct
         const int t = units[u].term;
         const uint32_t t_lo = ustart[(size_t)t * dp.n_groups], t_hi = ustart[(size_t)(t + 1) * dp.n_groups];
         const unsigned most = most_units(dp);
+        // a table becomes free when its last warp's unit ends: at most R
+        // unit_pair_bound pairs, 0.1 us each when all are rechecked
+        const unsigned long long limit = 4000000000ull + 100ull * R * dp.unit_pair_bound, since = gtimer();
 #pragma unroll 1
-        for (unsigned i = 0; i < (1u << 24) && k < 0; i++) {
+        while (k < 0 && gtimer() - since < limit) {
             if (!sched_lock(q)) break;
 #pragma unroll 1
-            for (int j = 0; j < dp.NT; j++)
-                if (q.term[j] == t && atomicAdd(&q.n_used[j], 1u) < most) k = j;
+            for (int j = 0; j < dp.NT; j++)   // a full table is not counted on: its counter could wrap
+                if (q.term[j] == t && *(volatile unsigned *)&q.n_used[j] < most && atomicAdd(&q.n_used[j], 1u) < most)
+                    k = j;
             if (k >= 0) {
                 q.ref[k]++;
             } else {

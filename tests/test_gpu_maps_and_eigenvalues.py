@@ -80,3 +80,24 @@ def test_eigvalsh_edges(tp, ctx, n, kind):
     ref = np.linalg.eigvalsh(C)
     assert np.all(np.diff(w) >= 0.0)
     assert np.max(np.abs(w - ref)) <= 8.0 * n * 2.0 ** -53 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 40, 120, 629])
+def test_eigvalsh_not_finite(tp, ctx, n):
+    """A NaN or an infinity in the matrix gives NaN eigenvalues, as on a matrix of NaNs."""
+    rng = np.random.default_rng(n)
+    a = rng.standard_normal((2 * n, n))
+    for value in (np.nan, np.inf):
+        for at in ((n - 1, n - 1), (0, n - 1), slice(None)):
+            C = a.T @ a
+            C[at] = value
+            if isinstance(at, tuple):
+                C[at[::-1]] = value
+            assert np.all(np.isnan(ctx.tpcf_eigvalsh(_dev(C)).cpu().numpy())), (value, at)
+
+
+def test_eigvalsh_of_a_diagonal_far_below_its_norm(tp, ctx):
+    """Entries 2^-80 of a diagonal matrix's norm come back to 2^-88 of the norm (e^2 is held above 2^-180)."""
+    d = np.array([1.0, 0.0, 2.0 ** -80, 2.0 ** -80, 3.0 * 2.0 ** -80, 0.0, 0.5, 2.0 ** -40])
+    w = ctx.tpcf_eigvalsh(_dev(np.diag(d))).cpu().numpy()
+    assert np.max(np.abs(w[:5] - np.sort(d)[:5])) <= 2.0 ** -88
