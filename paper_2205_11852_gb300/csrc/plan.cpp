@@ -411,9 +411,12 @@ bool build_direct(const tpcf_binning &b, const Plan &pl, int smem_sm, int smem_b
     // side: in a periodic box every neighbour within the last edge must lie
     // within half a box of the unit's corner (coordinates are differences from
     // it, modulo the box), and no cell may be a neighbour from both sides
-    if (group > 1 && b.geometry == TPCF_PERIODIC) {
-        const double smax_q = std::sqrt((double)p.T[b.n_s]) + 2.0;
-        if (!(group * Wmax + smax_q < std::ldexp(1.0, 31)) || group + 2 * pl.K > p.n_c) return false;
+    // (both hold for one cell at subdivision 2 and above; three cells, at
+    // subdivision 1 and last edges beyond a quarter of the box, fail the first)
+    if (b.geometry == TPCF_PERIODIC) {
+        const double reach = group * std::ceil(std::ldexp(1.0, p.bits) / p.n_c) - 1.0 +
+                             std::floor(std::sqrt((double)(p.T[b.n_s] - 1)));
+        if (!(reach < std::ldexp(1.0, 31)) || group + 2 * pl.K > p.n_c) return false;
     }
     d.G = group;
     d.n_groups = p.n_c * p.n_c * ((p.n_c + group - 1) / group);
