@@ -414,8 +414,8 @@ int tpcf_set_cell_subdiv(tpcf_ctx *ctx, int subdiv);
  *                        it.
  *   TPCF_OPT_KERNEL   -- which pair counter runs: TPCF_KERNEL_DIRECT (the
  *                        direct counter wherever the binning suits it -- s bins
- *                        linear from 0 with the x line of sight or s only, and
- *                        a histogram that fits shared memory with its copies --
+ *                        linear from 0, or geometric with the x line of sight
+ *                        or s only, and a histogram that fits shared memory --
  *                        else the general one), TPCF_KERNEL_GENERAL (always the
  *                        general counter) or TPCF_KERNEL_AUTO (the default: the
  *                        autotuner times both and keeps the faster; without a

@@ -396,13 +396,26 @@ bool build_direct(const tpcf_binning &b, const Plan &pl, int smem_sm, int smem_b
 {
     const CountParams &p = pl.prm;
     std::memset(&d, 0, sizeof(d));
-    if (!p.linear) return false;
     const bool mu = p.n_mu > 1;
     const bool mid = mu && p.los == TPCF_LOS_MIDPOINT;
     if (mu && p.los != TPCF_LOS_X && !mid) return false;
     const double L = b.box_L;
     const double q = std::ldexp(1.0, p.bits) / L;
-    const double qds = q * b.s_edges[1];
+    // geometric bins: unit u = e_0 / ratio, so that the edges lie at la
+    // log2(s^2 / u^2) = k + 1; dev: how far the exact thresholds are from that
+    const bool geo = !p.linear;
+    double unit = b.s_edges[geo ? 0 : 1], la = 0.0, dev = 0.0;
+    if (geo) {
+        if (mid || !(p.T[0] >= 1ull)) return false;
+        const double lr = std::log2(b.s_edges[b.n_s] / b.s_edges[0]) / b.n_s;   // log2 of the ratio
+        if (!(lr > 0.0)) return false;
+        unit *= std::exp2(-lr);
+        la = 0.5 / lr;
+        for (int k = 0; k <= b.n_s; k++)
+            dev = std::max(dev, std::fabs(la * (std::log2((double)p.T[k]) - 2.0 * std::log2(q * unit)) - (k + 1)));
+        dev += 1e-12 * b.n_s;
+    }
+    const double qds = q * unit;
     const float inv = (float)(1.0 / qds);
     const double u24 = std::ldexp(1.0, -24);
     const double kappa = std::fabs((double)inv * qds - 1.0);
@@ -423,11 +436,14 @@ bool build_direct(const tpcf_binning &b, const Plan &pl, int smem_sm, int smem_b
     const double Xg = (double)(pl.K + group) * Wmax;
     const double Xb = Xg / qds * (1.0 + std::ldexp(1.0, -20));
     const double E = 0.5 * ulp_f32(Xg) / qds * (1.0 + std::ldexp(1.0, -20)) + 0.5 * ulp_f32(Xb);
-    const double n_s = p.n_s, n_mu = p.n_mu;
-    const double e_d = 2.0 * E + 0.5 * ulp_f32(n_s + 2.0);
+    // Xs: the last edge in units; FAR, the padding points' place, must lie beyond it from any a-point
+    const double Xs = geo ? std::sqrt((double)p.T[b.n_s]) / qds * (1.0 + std::ldexp(1.0, -20)) : (double)p.n_s;
+    if (geo && !(Xs + Xb < 4.0e4)) return false;
+    const double n_mu = p.n_mu;
+    const double e_d = 2.0 * E + 0.5 * ulp_f32(Xs + 2.0);
     const double g3 = 3.0 * u24 / (1.0 - 3.0 * u24);
     const double rho = std::pow(2.0, -22.5);
-    const double dsq = 1.01 * (std::sqrt(3.0) * e_d + 3.0 * e_d * e_d + g3 * (n_s + 2.0) / 1.99);
+    const double dsq = 1.01 * (std::sqrt(3.0) * e_d + 3.0 * e_d * e_d + g3 * (Xs + 2.0) / 1.99);
     // mu margin (below) and the d2 addend: s only, a negligible 2^-60; with mu
     // bins, tiny = m0^2 / n_mu, which biases r = rsqrt(d2 + tiny) low by at
     // most n_mu tiny / (2 s) <= m0 / 4 in the mu interval for s >= 2 m0, and
@@ -461,12 +477,40 @@ bool build_direct(const tpcf_binning &b, const Plan &pl, int smem_sm, int smem_b
         if (!(d.c1 < 0.05f) || !(d.c3 < 0.05f) || !(d.c05 > 0.45f) || !(d.tinyl >= 1.0e-30f)) return false;
         m0 = c1_0 / n_mu;   // tiny = (c1_0 / n_mu)^2 below
     } else if (mu) {
-        m0 = 1.1 * (n_mu * 2.0 * E + 1.5 * ulp_f32(n_mu * Xb + 1.0) + n_mu * rho * (n_s + 1.0) + n_mu * dsq);
+        m0 = 1.1 * (n_mu * 2.0 * E + 1.5 * ulp_f32(n_mu * Xb + 1.0) + n_mu * rho * (Xs + 1.0) + n_mu * dsq);
         if (!(m0 < 0.04)) return false;
     }
     const float tiny = mid ? down_f(m0 * m0) : (mu ? down_f(m0 * m0 / n_mu) : (float)std::ldexp(1.0, -60));
     if (!(tiny > 0.0f)) return false;
-    const double eps_s = 1.1 * (dsq + rho * (n_s + 1.5) + kappa * (n_s + 1.0) + (double)tiny) + u24;
+    double eps_s = 1.1 * (dsq + rho * (Xs + 1.5) + kappa * (Xs + 1.0) + (double)tiny) + u24;
+    if (geo) {
+        // l = log2(d2): the relative error of d2 at s >= s_m (coordinates, rounding, the scale, the addend) times
+        // la / ln 2, lg2.approx's 2^-22 (absolute in (1/2, 2), relative elsewhere), la's rounding, the edges' own
+        // deviation and the residual's rounding.  s_m: the clamp's place (see pairdirect.cu); a pair below it by
+        // half a bin or more is not certain, or certain to miss.  Chosen: the clamp (0: half a bin above u) that
+        // leaves fewest pairs to recheck, with pairs uniform in volume.
+        auto eps_at = [&](double s_m) {
+            const double rel = 2.0 * std::sqrt(3.0) * e_d / s_m + 3.0 * e_d * e_d / (s_m * s_m) + g3 + 2.0 * kappa +
+                               (double)tiny / (s_m * s_m);
+            return 1.1 * (la / std::log(2.0) * 1.01 * rel +
+                          la * std::ldexp(1.0, -22) * std::max(1.0, 2.0 * std::log2(Xs + 2.0)) +
+                          (p.n_s + 2.0) * u24 + dev) + u24;
+        };
+        double best = 1e30;
+        int km = 0;
+        for (int k = 0; k < p.n_s; k++) {
+            const double e = eps_at(k == 0 ? 1.0 : std::exp2((k - 0.5) / (2.0 * la)));
+            const double rate = 2.0 * e + (k == 0 ? 0.0 : std::pow(std::exp2(k / (2.0 * la)) / Xs, 3.0));
+            if (e < 0.05 && rate < best) {
+                best = rate;
+                eps_s = e;
+                km = k;
+            }
+        }
+        if (!(best < 0.02)) return false;
+        d.la = (float)la;
+        d.lmid = (float)((km == 0 ? 0.5 : (double)km) / la);
+    }
     if (!(eps_s < 0.05)) return false;
     d.cs = down_f(0.5 - eps_s);
     d.logC = 0;
@@ -487,13 +531,16 @@ bool build_direct(const tpcf_binning &b, const Plan &pl, int smem_sm, int smem_b
     d.tiny = tiny;
     d.inv_qds = inv;
     d.nmu = (float)p.n_mu;
-    d.hit = up_f((n_s + 0.01) * (n_s + 0.01));
+    // (geometric bins: coordinates are larger, and so are their errors)
+    d.hit = geo ? up_f((Xs * 1.001 + 0.01) * (Xs * 1.001 + 0.01)) : up_f((Xs + 0.01) * (Xs + 0.01));
     // every pair's d2 is at least tiny, a normal float, so r = rsqrt(d2) is
     // finite and every histogram address stays inside the table
     if (!(d.tiny >= 1.0e-30f) || !std::isfinite(d.m) || !(d.cs > 0.4f) || !(inv > 0.0f)) return false;
-    d.s_top = (float)(8388608.0 + n_s);
     d.C = 1 << d.logC;
-    d.rows = p.n_s + 1;
+    d.geo = geo ? 1 : 0;
+    d.row0 = geo ? 1 : 0;
+    d.rows = d.row0 + p.n_s + 1;
+    d.s_top = (float)(8388608.0 + (d.rows - 1));
     // one block of DIRECT_WARPS warps per SM (their registers fill the
     // register file).  At least two tables, so that its warps pass from term to
     // term without waiting for each other, before copies (see pairdirect.cu);
@@ -506,7 +553,7 @@ bool build_direct(const tpcf_binning &b, const Plan &pl, int smem_sm, int smem_b
     for (const auto &op : opts) {
         if (!mu && op.R != 32) continue;
         if ((op.R == 32 && d.logC > 5) || (op.R == 8 && d.logC < 5)) continue;
-        const long long need = (long long)pairdirect_smem_bytes(p, op.R, d.C, op.NT, W);
+        const long long need = (long long)pairdirect_smem_bytes(p, d.rows, op.R, d.C, op.NT, W);
         if (need > budget) continue;
         d.NT = op.NT;
         d.R = op.R;

@@ -21,8 +21,9 @@ struct Plan {
 
 bool exact_threshold(double e, double L, int bits, unsigned long long &T);
 // Constants of the direct pair counter for a built plan; false when the
-// binning does not suit it (s bins not linear from 0, a midpoint line of
-// sight with mu bins, a histogram beyond shared memory, FP32 bands too wide).
+// binning does not suit it (s bins neither linear from 0 nor, with the x line
+// of sight or s only, geometric; a histogram beyond shared memory; FP32 bands
+// too wide).
 // smem_sm / smem_block: the device's shared memory per SM and per block
 // (opt-in), reserved: the per-block reservation.  group: cells along x that
 // share a unit; false when the periodic box is too small for it.

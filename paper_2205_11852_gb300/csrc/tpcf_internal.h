@@ -80,10 +80,9 @@ struct CountParams {
                                              // entry n_s+1 is +inf
 };
 
-// Constants of the direct pair counter (pairdirect.cu): linear s bins from 0
-// with the x line of sight or s only.  Every coordinate it handles is in
-// units of one s bin, relative to the integer lower corner of the unit's
-// cell; the error bounds behind m, cs and d2min are derived in plan.cpp.
+// Constants of the direct pair counter (pairdirect.cu).  Every coordinate it
+// handles is in units of one s bin (geometric bins: of the edge one bin below
+// the first), relative to the integer lower corner of the unit's cell; the error bounds behind m, cs and d2min are derived in plan.cpp.
 struct DirectParams {
     int R;             // histogram copies (lane l adds to copy l mod R)
     int NT;            // tables (terms) a block counts at a time, 1 to DIRECT_TABLES
@@ -91,7 +90,9 @@ struct DirectParams {
     int C;             // histogram columns, 1 << logC: signed mu columns from -CO, or 1 (s only)
     int logC;
     int CO;            // column of mu bin 0 (the signed mu bin j sits in column j + CO)
-    int rows;          // n_s + 1: the last row takes every pair at or beyond the last edge
+    int rows;          // row0 + n_s + 1: the last row takes every pair at or beyond the last edge
+    int row0;          // row of s bin 0: 1 for geometric bins (row 0: below the first edge), else 0
+    int geo;           // 1: geometric s bins
     int smem;          // dynamic shared memory bytes
     int mid;           // 1: mu from the midpoint line of sight
     unsigned long long unit_pair_bound;   // pairs one unit can add to one histogram counter
@@ -101,7 +102,8 @@ struct DirectParams {
     float cs;          // s residual bound: floor(u) is the bin when |u - floor(u) - 1/2| <= cs
     float tiny;        // d2 addend (keeps rsqrt finite; with mu bins it also bounds r)
     float hit;         // filter: squared box distance (bin^2) below which a b-point is kept
-    float s_top;       // 2^23 + n_s: the clamped row of pairs beyond the last edge
+    float s_top;       // 2^23 + rows - 1: the clamped row of pairs beyond the last edge
+    float la, lmid;    // geometric bins: row floor(la max(log2(d2), lmid))
     int G;             // cells along x that share a unit
     int n_groups;      // groups of cells per catalogue: n_c^2 ceil(n_c / G)
     // midpoint line of sight: t = n_mu mu is certain when |t - floor(t) - 1/2| <= c05 - c1 r - c3 rl
@@ -167,7 +169,7 @@ constexpr int DIRECT_TABLES = 4;     // histogram tables per block, at most
 cudaError_t launch_pairdirect(const CountParams &p, const DirectParams &d, const Mesh &m, const Term *terms,
                               const Unit *units, const uint32_t *ustart, const uint32_t *n_units, unsigned *claim,
                               unsigned long long *stats, int *status, const PairLaunch &pl, cudaStream_t s);
-size_t pairdirect_smem_bytes(const CountParams &p, int R, int C, int NT, int W);
+size_t pairdirect_smem_bytes(const CountParams &p, int rows, int R, int C, int NT, int W);
 cudaError_t pairdirect_set_attrs(const DirectParams &d, int mu);
 int pairdirect_max_blocks_per_sm(const DirectParams &d, int mu);
 
