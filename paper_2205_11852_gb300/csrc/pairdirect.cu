@@ -52,6 +52,15 @@
 // 100 000 points, 24 bins from 0.75 to 150 Mpc/h: 4.81 ms by the general counter, 3.04 so
 // (eight pairs in 10^4 rechecked).
 //
+// Fine mu bins along x (the signed table of mode 1 would not fit): one copy of a
+// table with a column per |mu| bin, T from |n_mu dx|, rows a whole number of
+// columns apart.  Two lanes seldom meet in one of so many bins, and the
+// banks they fall in are as good as random (about three adds in the fullest).
+// T- below column -1 only occurs in row 0 and only for uncertain pairs, whose
+// adds are taken back: FOLD_PAD words before the table take them.
+// 155 250 points in a slab, 200 x 100 bins: 13.06 ms by the general counter, 6.78 so
+// (one table per block; 10 pairs in 10^4 rechecked).
+//
 // Histogram.  R copies of a (n_s + 1) x C table of 32-bit counters, lane l
 // adding to copy l mod R, so the 32 adds of a warp fall in distinct banks
 // (R = 32) or at most two per bank (R = 16).  mu is binned by sign, C =
@@ -90,6 +99,7 @@ struct Sched {
     unsigned ref[MAX_NT];       // warps adding to a table
 };
 constexpr int FREE = -1, DRAINING = -2;
+constexpr int FOLD_PAD = DIRECT_FOLD_PAD;   // words before a table of one copy (mode 5)
 
 // Shared memory: the block's one or two tables, T, the schedule, then one
 // region per warp: a-records (3 float4 per a-point), the b buffer (float4: x, y, z in
@@ -104,7 +114,7 @@ __host__ __device__ inline DOff d_off(int n_s, int rows, int n_rows, int R, int 
 {
     DOff o;
     o.hist = 0;
-    o.hstride = al16(4u * (uint32_t)(rows * C * R));
+    o.hstride = al16(4u * (uint32_t)(rows * C * R + (R == 1 ? FOLD_PAD : 0)));
     o.T = o.hstride * (uint32_t)NT;
     o.misc = al16(o.T + 8u * (uint32_t)(n_s + 1));
     o.warp0 = o.misc + al16((uint32_t)sizeof(Sched));
@@ -135,26 +145,29 @@ struct ARec {
 // Histogram address of a pair with s-row word bits(S) and signed-mu-column
 // word bits(T-): (bits(S) << LS) + (bits(T-) << LT) + Kl, with LT = log2(4 R)
 // and LS = LT + log2(C), so that the row and column strides are shifts.
+// With one copy (mode 5) a row is 4 C bytes, multiplied instead of shifted.
 template <int R, int LOGC>
 struct Sh {
-    static constexpr int LT = R == 32 ? 7 : (R == 16 ? 6 : (R == 8 ? 5 : -1));
+    static constexpr int LT = R == 32 ? 7 : (R == 16 ? 6 : (R == 8 ? 5 : (R == 1 ? 2 : -1)));
     static constexpr int LS = LT + LOGC;
-    static_assert(LT > 0, "R is 8, 16 or 32");
+    static_assert(LT > 0, "R is 1, 8, 16 or 32");
 };
 
 __device__ __forceinline__ uint64_t u64of(float2 v) { return *reinterpret_cast<uint64_t *>(&v); }
 
 // Constant operand pairs of the packed arithmetic (tinyl to c05: midpoint
-// line of sight only; la and the clamp lmid: geometric s bins only).
+// line of sight only; la and the clamp lmid: geometric s bins only; mm = m and
+// the row's bytes rs: mode 5 only).
 struct K2 {
-    uint64_t tiny, ms, m1, mh, mt, nm, tinyl, mhalf, c1n, c3n, c05, la;
+    uint64_t tiny, ms, m1, mh, mt, nm, tinyl, mhalf, c1n, c3n, c05, la, mm;
     float lmid;
+    uint32_t rs;
 };
 
 // The kernel's modes V: 0 s only, 1 mu along x, 2 mu from the midpoint; 3 and
-// 4 are 0 and 1 with geometric s bins.
-__host__ __device__ constexpr bool has_mu(int V) { return V == 1 || V == 2 || V == 4; }
-__host__ __device__ constexpr bool is_geo(int V) { return V >= 3; }
+// 4 are 0 and 1 with geometric s bins; 5 is 1 with one column per |mu| bin.
+__host__ __device__ constexpr bool has_mu(int V) { return V != 0 && V != 3; }
+__host__ __device__ constexpr bool is_geo(int V) { return V == 3 || V == 4; }
 
 // One packed pair of pairs (b_p, a), (b_p', a) in hand-written PTX: the
 // packed s floor word S and s residual FS (the tiny addend, r = rsqrt(d2) by
@@ -242,6 +255,34 @@ __device__ __forceinline__ void pair2_core(uint64_t bx, uint64_t by, uint64_t bz
               "l"(u64of(a.q)), "l"(k.tiny), "l"(k.ms), "l"(k.m1), "l"(k.mh), "l"(k.mt), "l"(k.nm), "l"(k.la),
               "f"(k.lmid));
         CB = 0;
+    } else if (V == 5) {
+        asm("{\n\t"
+            ".reg .b64 dx, dy, dz, d2, r, h, x, xp, xm;\n\t"
+            ".reg .f32 d2x, d2y, rx, ry;\n\t"
+            "add.rn.f32x2 dx, %4, %7;\n\t"
+            "add.rn.f32x2 dy, %5, %8;\n\t"
+            "add.rn.f32x2 dz, %6, %9;\n\t"
+            "fma.rn.f32x2 d2, dx, dx, %11;\n\t"
+            "fma.rn.f32x2 d2, dy, dy, d2;\n\t"
+            "fma.rn.f32x2 d2, dz, dz, d2;\n\t"
+            "mov.b64 {d2x, d2y}, d2;\n\t"
+            "rsqrt.approx.ftz.f32 rx, d2x;\n\t"
+            "rsqrt.approx.ftz.f32 ry, d2y;\n\t"
+            "mov.b64 r, {rx, ry};\n\t"
+            "fma.rz.f32x2 %0, d2, r, %12;\n\t"
+            "fma.rn.f32x2 h, %0, %13, %14;\n\t"
+            "fma.rn.f32x2 %1, d2, r, h;\n\t"
+            "fma.rn.f32x2 x, %4, %16, %10;\n\t"
+            "and.b64 x, x, 0x7fffffff7fffffff;\n\t"
+            "add.rn.f32x2 xp, x, %17;\n\t"
+            "fma.rn.f32x2 xm, %17, %13, x;\n\t"
+            "fma.rz.f32x2 %2, xp, r, %15;\n\t"
+            "fma.rz.f32x2 %3, xm, r, %15;\n\t"
+            "}"
+            : "=&l"(S), "=&l"(FS), "=&l"(TP), "=&l"(TM)
+            : "l"(bx), "l"(by), "l"(bz), "l"(u64of(a.nax)), "l"(u64of(a.nay)), "l"(u64of(a.naz)), "l"(u64of(a.p)),
+              "l"(k.tiny), "l"(k.ms), "l"(k.m1), "l"(k.mh), "l"(k.mt), "l"(k.nm), "l"(k.mm));
+        CB = 0;
     } else if (V == 3) {
         asm("{\n\t"
             ".reg .b64 dx, dy, dz, d2, l, h;\n\t"
@@ -322,13 +363,14 @@ __device__ __forceinline__ float hi_f(uint64_t v) { return __uint_as_float((uint
 
 // Histogram addresses of the two pairs: the s row (S clamped to the spare
 // last row) and, with mu bins, the signed mu column of T-.
-template <bool MU, int LS, int LT>
-__device__ __forceinline__ void pair_addr(uint64_t S, uint64_t TM, float stop, uint32_t Kl, uint32_t &a0,
+template <int V, int LS, int LT>
+__device__ __forceinline__ void pair_addr(uint64_t S, uint64_t TM, float stop, uint32_t Kl, uint32_t rs, uint32_t &a0,
                                           uint32_t &a1)
 {
-    a0 = Kl + (__float_as_uint(fminf(lo_f(S), stop)) << LS);
-    a1 = Kl + (__float_as_uint(fminf(hi_f(S), stop)) << LS);
-    if (MU) {
+    const uint32_t s0 = __float_as_uint(fminf(lo_f(S), stop)), s1 = __float_as_uint(fminf(hi_f(S), stop));
+    a0 = Kl + (V == 5 ? s0 * rs : s0 << LS);
+    a1 = Kl + (V == 5 ? s1 * rs : s1 << LS);
+    if (has_mu(V)) {
         a0 += (uint32_t)TM << LT;
         a1 += (uint32_t)(TM >> 32) << LT;
     }
@@ -344,10 +386,10 @@ __device__ __forceinline__ void pair2_flags(uint64_t bx, uint64_t by, uint64_t b
 {
     uint64_t S, FS, TP, TM, CB;
     pair2_core<V>(bx, by, bz, a, k, S, FS, TP, TM, CB);
-    pair_addr<has_mu(V), LS, LT>(S, TM, stop, Kl, a0, a1);
+    pair_addr<V, LS, LT>(S, TM, stop, Kl, k.rs, a0, a1);
     f0 = fabsf(lo_f(FS)) > cs;
     f1 = fabsf(hi_f(FS)) > cs;
-    if (V == 1 || V == 4) {
+    if (V == 1 || V == 4 || V == 5) {
         f0 = f0 || lo_f(TP) != lo_f(TM);
         f1 = f1 || hi_f(TP) != hi_f(TM);
     } else if (V == 2) {
@@ -364,7 +406,8 @@ __device__ __forceinline__ void pair2_flags(uint64_t bx, uint64_t by, uint64_t b
 // cell): a pair with a >= b goes to the lane's spare word instead.
 // Operands: %0 the lane's uncertainty; %1-%6 b (x, y, z) of q = 0, 1; %7-%11 the a-record;
 // %12-%17 constants; %18 cs; %19 the s clamp; %20 Kl; %21, %22 LS, LT;
-// CHK: %23 a index, %24-%27 b indices of slots 0-3, %28 spare word; geometric bins: A and lmid after these.
+// CHK: %23 a index, %24-%27 b indices of slots 0-3, %28 spare word; geometric bins: A and lmid after these, mode 5: m and
+// a row's bytes.
 #define PD_D2(BX, BY, BZ)                            \
     "add.rn.f32x2 dx, " BX ", %7;\n\t"                 \
     "add.rn.f32x2 dy, " BY ", %8;\n\t"                 \
@@ -400,16 +443,26 @@ __device__ __forceinline__ void pair2_flags(uint64_t bx, uint64_t by, uint64_t b
     "min.f32 sx, sx, %19;\n\t"                         \
     "min.f32 sy, sy, %19;\n\t"                         \
     "mov.b32 ux, sx;\n\t"                              \
-    "mov.b32 uy, sy;\n\t"                              \
+    "mov.b32 uy, sy;\n\t"
+#define PD_ROW                                       \
     "shl.b32 ux, ux, %21;\n\t"                         \
     "shl.b32 uy, uy, %21;\n\t"                         \
     "add.u32 ux, ux, %20;\n\t"                         \
     "add.u32 uy, uy, %20;\n\t"
-#define PD_DIFF(BX, BY, BZ) PD_D2(BX, BY, BZ) PD_RSQ PD_LIN PD_S
-#define PD_GEO(BX, BY, BZ, LA, LMID) PD_D2(BX, BY, BZ) PD_LG2(LA, LMID) PD_S
+#define PD_DIFF(BX, BY, BZ) PD_D2(BX, BY, BZ) PD_RSQ PD_LIN PD_S PD_ROW
+#define PD_GEO(BX, BY, BZ, LA, LMID) PD_D2(BX, BY, BZ) PD_LG2(LA, LMID) PD_S PD_ROW
+#define PD_ABS(BX, BY, BZ, MM, RS)                   \
+    PD_D2(BX, BY, BZ) PD_RSQ PD_LIN PD_S               \
+    "mad.lo.u32 ux, ux, " RS ", %20;\n\t"              \
+    "mad.lo.u32 uy, uy, " RS ", %20;\n\t"              \
+    "fma.rn.f32x2 xm, " BX ", %17, %10;\n\t"           \
+    "and.b64 xm, xm, 0x7fffffff7fffffff;\n\t"          \
+    "add.rn.f32x2 xp, xm, " MM ";\n\t"                 \
+    "fma.rn.f32x2 xm, " MM ", %14, xm;\n\t" PD_COL
 #define PD_MU(BX)                                    \
     "fma.rn.f32x2 xp, " BX ", %17, %10;\n\t"           \
-    "fma.rn.f32x2 xm, " BX ", %17, %11;\n\t"           \
+    "fma.rn.f32x2 xm, " BX ", %17, %11;\n\t" PD_COL
+#define PD_COL                                       \
     "fma.rz.f32x2 tp, xp, r, %16;\n\t"                 \
     "fma.rz.f32x2 tm, xm, r, %16;\n\t"                 \
     "mov.b64 {px, py}, tp;\n\t"                        \
@@ -560,7 +613,20 @@ __device__ __forceinline__ bool apoint(const float2 (&BX)[NQ], const float2 (&BY
         "l"(u64of(BZ[1])), "l"(u64of(a.nax)), "l"(u64of(a.nay)), "l"(u64of(a.naz)), "l"(u64of(a.p)),             \
         "l"(u64of(a.q)), "l"(k.tiny), "l"(k.ms), "l"(k.m1), "l"(k.mh), "l"(k.mt), "l"(k.nm), "f"(cs), "f"(stop), \
         "r"(Kl), "n"(LS), "n"(LT)
-    if (V == 4 && CHK) {
+    if (V == 5 && CHK) {
+        asm volatile(PD_HEAD PD_ABS("%1", "%2", "%3", "%29", "%30") PD_CHK("%24", "%25") PD_RED
+                         PD_ABS("%4", "%5", "%6", "%29", "%30") PD_CHK("%26", "%27") PD_RED PD_TAIL
+                     : "=r"(any)
+                     : PD_IN, "r"(ia), "r"(IB[0]), "r"(IB[1]), "r"(IB[2]), "r"(IB[3]), "r"(dump), "l"(k.mm),
+                       "r"(k.rs)
+                     : "memory");
+    } else if (V == 5) {
+        asm volatile(PD_HEAD PD_ABS("%1", "%2", "%3", "%23", "%24") PD_RED PD_ABS("%4", "%5", "%6", "%23", "%24")
+                         PD_RED PD_TAIL
+                     : "=r"(any)
+                     : PD_IN, "l"(k.mm), "r"(k.rs)
+                     : "memory");
+    } else if (V == 4 && CHK) {
         asm volatile(PD_HEAD PD_GEO("%1", "%2", "%3", "%29", "%30") PD_RSQ PD_MU("%1") PD_CHK("%24", "%25") PD_RED
                          PD_GEO("%4", "%5", "%6", "%29", "%30") PD_RSQ PD_MU("%4") PD_CHK("%26", "%27") PD_RED PD_TAIL
                      : "=r"(any)
@@ -620,6 +686,9 @@ __device__ __forceinline__ bool apoint(const float2 (&BX)[NQ], const float2 (&BY
 #undef PD_S
 #undef PD_DIFF
 #undef PD_GEO
+#undef PD_ROW
+#undef PD_ABS
+#undef PD_COL
 #undef PD_MU
 #undef PD_CHK
 #undef PD_RED
@@ -638,12 +707,18 @@ struct Addr {
     uint32_t Kl;
     __device__ __forceinline__ static uint32_t shift(const DirectParams &dp)
     {
+        if (R == 1) return 4u * (uint32_t)dp.CO - MAG_S_BITS * (4u * (uint32_t)dp.C) - (MAG_T_BITS << LT);
         return MU ? ((uint32_t)dp.CO << LT) - (MAG_S_BITS << LS) - (MAG_T_BITS << LT) : 0u - (MAG_S_BITS << LS);
+    }
+    // row k, column c from the base hb
+    __device__ __forceinline__ static uint32_t cell(const DirectParams &dp, uint32_t hb, uint32_t k, uint32_t c)
+    {
+        return hb + (R == 1 ? 4u * (k * (uint32_t)dp.C + c) : (k << LS) + (c << LT));
     }
     __device__ __forceinline__ uint32_t hb(const DirectParams &dp) const { return Kl - shift(dp); }
     __device__ __forceinline__ uint32_t dump(const DirectParams &dp) const
     {
-        return hb(dp) + ((uint32_t)(dp.rows - 1) << LS);
+        return cell(dp, hb(dp), (uint32_t)(dp.rows - 1), R == 1 ? (uint32_t)dp.CO : 0u);
     }
 };
 
@@ -697,7 +772,7 @@ __device__ __forceinline__ void recheck(const CountParams &prm, const DirectPara
         if (bin >= 0) {
             const uint32_t k = (uint32_t)bin / (uint32_t)prm.n_mu + (uint32_t)dp.row0, j = (uint32_t)bin % (uint32_t)prm.n_mu;
             const uint32_t col = MU ? j + (uint32_t)dp.CO : 0u;
-            red_add(hb + (k << Sh<R, LOGC>::LS) + (col << Sh<R, LOGC>::LT), 1u);
+            red_add(Addr<MU, R, LOGC>::cell(dp, hb, k, col), 1u);
         }
     }
     __syncwarp();
@@ -782,7 +857,9 @@ __device__ __forceinline__ void tile(const CountParams &prm, const DirectParams 
                 MID ? u64of(make_float2(-dp.c3, -dp.c3)) : 0ull,
                 MID ? u64of(make_float2(dp.c05, dp.c05)) : 0ull,
                is_geo(V) ? u64of(make_float2(dp.la, dp.la)) : 0ull,
-               is_geo(V) ? dp.lmid : 0.0f};
+               V == 5 ? u64of(make_float2(dp.m, dp.m)) : 0ull,
+               is_geo(V) ? dp.lmid : 0.0f,
+               V == 5 ? 4u * (uint32_t)dp.C : 0u};
     const uint32_t lt = (1u << lane) - 1u;
     // a-point ai had an uncertain pair in some lane: recompute its pairs with
     // one flag each (padding slots and, in the self cell, pairs a >= b never
@@ -885,7 +962,7 @@ __device__ __forceinline__ void unit(const CountParams &prm, const DirectParams 
             wm.arec[3 * i + 2] = make_float4(lay, lay, laz, laz);
         } else {
             const float fxp = __fmul_rn(p.x, dp.nmu);
-            const float cp = __fsub_rn(dp.m, fxp), cm = __fsub_rn(-dp.m, fxp);
+            const float cp = V == 5 ? -fxp : __fsub_rn(dp.m, fxp), cm = V == 5 ? 0.0f : __fsub_rn(-dp.m, fxp);
             wm.arec[3 * i + 1] = make_float4(-p.z, -p.z, cp, cp);
             wm.arec[3 * i + 2] = make_float4(cm, cm, 0.f, 0.f);
         }
@@ -1081,6 +1158,12 @@ __device__ __forceinline__ unsigned long long drain(const CountParams &prm, cons
     for (int b = lane; b < prm.nbin; b += 32) {
         const int k = b / n_mu + dp.row0, j = b % n_mu;
         unsigned long long sum = 0;
+        if (R == 1) {   // one copy, one column per |mu| bin
+            sum = hist[(uint32_t)k * (uint32_t)dp.C + (uint32_t)(j + dp.CO)];
+            if (sum) atomicAdd((unsigned long long *)&th[b], sum);
+            binned += sum;
+            continue;
+        }
         // mu bin j: signed columns j and -1 - j
         const uint32_t c1 = MU ? (uint32_t)(j + dp.CO) : 0u, c2 = MU ? (uint32_t)(dp.CO - 1 - j) : 0u;
         const uint4 *w1 = (const uint4 *)(hist + (((uint32_t)k << LOGC) + c1) * (uint32_t)R);
@@ -1372,6 +1455,7 @@ void *select_direct(int V, int R, int W, int logC)
 {
     if (W != DIRECT_WARPS) return nullptr;
     constexpr int DW = DIRECT_WARPS;
+    if (V == 5) return R == 1 ? dkernel<5, 1, DW, 0>() : nullptr;
     if (V == 3) return R == 32 ? dkernel<3, 32, DW, 0>() : nullptr;
     if (V == 4 && logC == 4) return R == 32 ? dkernel<4, 32, DW, 4>() : (R == 16 ? dkernel<4, 16, DW, 4>() : nullptr);
     if (V == 4 && logC == 5) return R == 32 ? dkernel<4, 32, DW, 5>() : (R == 16 ? dkernel<4, 16, DW, 5>() : dkernel<4, 8, DW, 5>());
@@ -1386,7 +1470,7 @@ void *select_direct(int V, int R, int W, int logC)
     return nullptr;
 }
 
-int mode_of(const DirectParams &d, bool mu) { return d.geo ? (mu ? 4 : 3) : (!mu ? 0 : (d.mid ? 2 : 1)); }
+int mode_of(const DirectParams &d, bool mu) { return d.R == 1 ? 5 : d.geo ? (mu ? 4 : 3) : (!mu ? 0 : (d.mid ? 2 : 1)); }
 
 }  // namespace
 

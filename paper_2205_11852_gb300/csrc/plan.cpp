@@ -525,7 +525,12 @@ bool build_direct(const tpcf_binning &b, const Plan &pl, int smem_sm, int smem_b
         int lc = 0;
         while ((1 << lc) < 2 * d.CO) lc++;
         if (lc < 4) lc = 4;
-        if (lc > 6) return false;
+        if (lc > 6) {
+            // too many signed columns: one per |mu| bin and one that takes T- = n_mu and the next row's T- = -1
+            if (mid || geo || (int)std::ceil(ext) > DIRECT_FOLD_PAD) return false;
+            d.CO = DIRECT_FOLD_PAD;
+            lc = -1;
+        }
         d.logC = lc;
     }
     d.tiny = tiny;
@@ -536,7 +541,7 @@ bool build_direct(const tpcf_binning &b, const Plan &pl, int smem_sm, int smem_b
     // every pair's d2 is at least tiny, a normal float, so r = rsqrt(d2) is
     // finite and every histogram address stays inside the table
     if (!(d.tiny >= 1.0e-30f) || !std::isfinite(d.m) || !(d.cs > 0.4f) || !(inv > 0.0f)) return false;
-    d.C = 1 << d.logC;
+    d.C = d.logC < 0 ? p.n_mu + 2 : 1 << d.logC;
     d.geo = geo ? 1 : 0;
     d.row0 = geo ? 1 : 0;
     d.rows = d.row0 + p.n_s + 1;
@@ -549,9 +554,10 @@ bool build_direct(const tpcf_binning &b, const Plan &pl, int smem_sm, int smem_b
     constexpr int W = DIRECT_WARPS;
     static const struct {
         int NT, R;
-    } opts[] = {{4, 32}, {2, 32}, {4, 16}, {2, 16}, {2, 8}, {1, 16}, {1, 8}};
+    } opts[] = {{4, 32}, {2, 32}, {4, 16}, {2, 16}, {2, 8}, {1, 16}, {1, 8}, {2, 1}, {1, 1}};
     for (const auto &op : opts) {
         if (!mu && op.R != 32) continue;
+        if ((op.R == 1) != (d.logC < 0)) continue;
         if ((op.R == 32 && d.logC > 5) || (op.R == 8 && d.logC < 5)) continue;
         const long long need = (long long)pairdirect_smem_bytes(p, d.rows, op.R, d.C, op.NT, W);
         if (need > budget) continue;

@@ -88,7 +88,7 @@ struct DirectParams {
     int NT;            // tables (terms) a block counts at a time, 1 to DIRECT_TABLES
     int W;             // warps per block (one block per SM)
     int C;             // histogram columns, 1 << logC: signed mu columns from -CO, or 1 (s only)
-    int logC;
+    int logC;          // -1: one column per |mu| bin, C of them (one copy)
     int CO;            // column of mu bin 0 (the signed mu bin j sits in column j + CO)
     int rows;          // row0 + n_s + 1: the last row takes every pair at or beyond the last edge
     int row0;          // row of s bin 0: 1 for geometric bins (row 0: below the first edge), else 0
@@ -166,6 +166,7 @@ int paircount_max_blocks_per_sm(const CountParams &p, int warps_per_block, int s
 constexpr int DIRECT_ACHUNK = 64;    // a-points per work unit
 constexpr int DIRECT_WARPS = 16;
 constexpr int DIRECT_TABLES = 4;     // histogram tables per block, at most
+constexpr int DIRECT_FOLD_PAD = 16;   // words before a table of one copy: columns -16 to -1 of row 0
 cudaError_t launch_pairdirect(const CountParams &p, const DirectParams &d, const Mesh &m, const Term *terms,
                               const Unit *units, const uint32_t *ustart, const uint32_t *n_units, unsigned *claim,
                               unsigned long long *stats, int *status, const PairLaunch &pl, cudaStream_t s);
