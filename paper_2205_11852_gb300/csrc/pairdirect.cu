@@ -904,8 +904,17 @@ __device__ __forceinline__ void tile(const CountParams &prm, const DirectParams 
         const bool u0 = apoint<V, CHK, LS, LT>(BX, BY, BZ, a, k2, dp.cs, dp.s_top, ad.Kl, a0 + ai, IB, dump);
         const bool u1 = apoint<V, CHK, LS, LT>(BX, BY, BZ, a2, k2, dp.cs, dp.s_top, ad.Kl, a0 + ai + 1, IB, dump);
         if (__any_sync(0xffffffffu, u0 || u1)) {
+            // rarely both a-points have an uncertain pair (fine mu bins 7.65 -> 7.14 ms, three mocks of a
+            // million points 60.7 -> 60.0); the midpoint kernel (33.55 -> 33.74) and linear s-only bins, which
+            // seldom come here (16 mocks of 100 000 points 9.24 -> 9.50), lose by the second vote
+            if (MID || V == 0) {
 #pragma unroll 1
-            for (uint32_t j = ai; j < ai + 2; j++) settle(j);
+                for (uint32_t j = ai; j < ai + 2; j++) settle(j);
+            } else {
+#pragma unroll 1
+                for (uint32_t j = 0; j < 2; j++)
+                    if (__any_sync(0xffffffffu, j ? u1 : u0)) settle(ai + j);
+            }
         }
     }
     if (ai < na) {   // the last a-point of an odd chunk
