@@ -430,8 +430,12 @@ int tpcf_lc_cov(tpcf_ctx *ctx, const double *xi_a1, const double *xi_a2, const d
     if (!(M >= (double)M_a)) return fail(ctx, TPCF_ERR_ARG, "M must be >= M_a (or +inf)");
     if (precision == TPCF_FP64) {
         void *w;
-        if (cov_digits_suits(n_mock, nbin, 3, ctx->n_sm)) {
-            if ((rc = ensure(ctx, "lc_digits_work", cov_digits_work_bytes(n_mock, nbin, 3, ctx->n_sm), &w))) return rc;
+        // (without room for its larger workspace the float64 kernel runs)
+        rc = TPCF_ERR_NOMEM;
+        if (cov_digits_suits(n_mock, nbin, 3, ctx->n_sm))
+            rc = ensure(ctx, "lc_digits_work", cov_digits_work_bytes(n_mock, nbin, 3, ctx->n_sm), &w);
+        if (rc && rc != TPCF_ERR_NOMEM) return rc;
+        if (!rc) {
             CK(launch_cov_digits(xi_a1, xi_a2, xi_b, 3, n_mock, nbin, w, ctx->n_sm, M_a, M, C_lc, Ca, Cb, A, B,
                                  ctx->status, s));
             return TPCF_OK;
@@ -464,8 +468,11 @@ int tpcf_sample_cov(tpcf_ctx *ctx, const double *xi, int n_mock, int nbin, int p
     if (nbin < 1 || nbin > 65536) return fail(ctx, TPCF_ERR_ARG, "bad nbin");
     if (precision == TPCF_FP64) {
         void *w;
-        if (cov_digits_suits(n_mock, nbin, 1, ctx->n_sm)) {
-            if ((rc = ensure(ctx, "lc_digits_work", cov_digits_work_bytes(n_mock, nbin, 1, ctx->n_sm), &w))) return rc;
+        rc = TPCF_ERR_NOMEM;
+        if (cov_digits_suits(n_mock, nbin, 1, ctx->n_sm))
+            rc = ensure(ctx, "lc_digits_work", cov_digits_work_bytes(n_mock, nbin, 1, ctx->n_sm), &w);
+        if (rc && rc != TPCF_ERR_NOMEM) return rc;
+        if (!rc) {
             CK(launch_cov_digits(xi, xi, xi, 1, n_mock, nbin, w, ctx->n_sm, 1, 2.0, C, nullptr, nullptr, nullptr,
                                  nullptr, ctx->status, s));
             return TPCF_OK;

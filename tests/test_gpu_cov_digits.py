@@ -91,3 +91,19 @@ def test_cov_digits_extreme_columns(tp, ctx):
     assert np.all(np.isnan(s[bad]))
     ok = [i for i in range(nb) if i not in (8, 9)]
     assert _norm_err(s[np.ix_(ok, ok)], ref[np.ix_(ok, ok)]) <= tol
+
+
+def test_cov_digits_without_room_for_the_workspace(tp, monkeypatch):
+    """A failed allocation of the digit workspace leaves the call to the float64 kernel and its smaller one."""
+    xs = synth.synthetic_xi_variants(62, 50, 30)
+    monkeypatch.setenv("TPCF_TEST_FAIL_ALLOC", "1")
+    ctx = tp.Context(0)
+    monkeypatch.delenv("TPCF_TEST_FAIL_ALLOC")
+    tol = 4.0 * 51 * 2.0 ** -53
+    ref = oracle.lc_cov(*xs, 1, 50.0)
+    d = np.sqrt(np.diag(ref["Ca"]))
+    for _ in range(2):   # the float64 kernel, then the digits
+        got = ctx.tpcf_lc_cov(*[_dev(x) for x in xs], 1, 50.0, tp.TPCF_FP64)["C_lc"].cpu().numpy()
+        assert ctx.tpcf_sync() == tp.TPCF_OK
+        assert float(np.max(np.abs(got - ref["C_lc"]) / np.outer(d, d))) <= 4.0 * tol
+    ctx.close()
