@@ -49,7 +49,7 @@
 // a whole number (a pair below that bin, where FP32 errors are large against
 // a bin, is always rechecked) or 1/2 (a pair that far below the first
 // edge is certain to miss), whichever leaves fewer pairs to recheck.  Three mocks of
-// 100 000 points, 24 bins from 0.75 to 150 Mpc/h: 4.81 ms by the general counter, 3.04 so
+// 100 000 points, 24 bins from 0.75 to 150 Mpc/h: 4.81 ms by the general counter, 2.98 so
 // (eight pairs in 10^4 rechecked).
 //
 // Fine mu bins along x (the signed table of mode 1 would not fit): one copy of a
@@ -58,7 +58,7 @@
 // banks they fall in are as good as random (about three adds in the fullest).
 // T- below column -1 only occurs in row 0 and only for uncertain pairs, whose
 // adds are taken back: FOLD_PAD words before the table take them.
-// 155 250 points in a slab, 200 x 100 bins: 13.06 ms by the general counter, 6.78 so
+// 155 250 points in a slab, 200 x 100 bins: 13.06 ms by the general counter, 6.28 so
 // (one table per block; 10 pairs in 10^4 rechecked).
 //
 // Histogram.  R copies of a (n_s + 1) x C table of 32-bit counters, lane l
