@@ -1007,7 +1007,7 @@ extern "C" int tpcf_count(tpcf_ctx *ctx, const tpcf_mock *mocks, int n_mock, con
         auto it = ctx->tune_cache.find(tune_key(ctx, mocks, n_mock, binning, terms));
         if (it != ctx->tune_cache.end()) cfg = it->second;
         // but for sparse catalogues' large units: a launch of one term has too few of them to fill the SMs
-        // (16 mocks of 4000 points, whole step: 5.1 ms at subdivision 1, 3.7 at 2)
+        // (16 mocks of 4000 points, whole step: 5.1 ms at subdivision 1, 3.3 at 2)
         if (cfg.subdiv < 2) cfg.subdiv = 2;
         cfg.group = 1;
     } else if (ctx->autotune && mode == TPCF_BATCHED && n_mock > 0) {
