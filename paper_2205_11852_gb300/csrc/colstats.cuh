@@ -14,26 +14,25 @@ namespace {
 constexpr int COL_WARPS = 8;      // warps per block, interleaved over the rows; lane = column
 constexpr int COL_CHUNKS = 32;    // row ranges per column block
 
-// The extrema are kept as order-preserving keys of the doubles' upper words
-// (integer minima; the float64 pipe, two operations per clock and SM, is left
-// to the sums), widened to the next upper word when they are read back.
+// The extrema are kept as order-preserving integer keys of the doubles
+// (integer minima: the float64 pipe, two operations per clock and SM, is left
+// to the sums).  All 64 bits: a column's scatter can be far below its mean,
+// and extrema known to 2^-20 of their value only would bound the residuals of
+// such a column by 2^-20 of the mean.
 struct ColPartial {
     double sum;
-    int lo, hi;
+    long long lo, hi;
 };
+constexpr long long KEY_MAX = 0x7fffffffffffffffll;
 
-__device__ __forceinline__ int key_of(double v)
+__device__ __forceinline__ long long key_of(double v)
 {
-    const int h = __double2hiint(v);
-    return h ^ ((h >> 31) & 0x7fffffff);
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & KEY_MAX);
 }
 
-// a bound of every double with the key: the smallest (up = false) or the largest one
-__device__ __forceinline__ double key_bound(int key, bool up)
-{
-    const int h = key ^ ((key >> 31) & 0x7fffffff);
-    return __hiloint2double(h, (h < 0) == up ? 0 : -1);
-}
+// the double with the key
+__device__ __forceinline__ double of_key(long long key) { return __longlong_as_double(key ^ ((key >> 63) & KEY_MAX)); }
 
 // part[v][chunk][b] of the rows [chunk * per, (chunk + 1) * per)
 __global__ void __launch_bounds__(32 * COL_WARPS)
@@ -47,7 +46,7 @@ __global__ void __launch_bounds__(32 * COL_WARPS)
     const int per = (n_mock + COL_CHUNKS - 1) / COL_CHUNKS;
     const int m0 = min(n_mock, (int)blockIdx.y * per), m1 = min(n_mock, m0 + per);
     double s[2] = {0.0, 0.0};
-    int lo = 0x7fffffff, hi = -0x7fffffff - 1;
+    long long lo = KEY_MAX, hi = -KEY_MAX - 1;
     if (b < nbin) {
         int m = m0 + warp;
         constexpr int U = 8;
@@ -57,17 +56,19 @@ __global__ void __launch_bounds__(32 * COL_WARPS)
             for (int k = 0; k < U; k++) t[k] = x[(size_t)(m + k * COL_WARPS) * nbin + b];
 #pragma unroll
             for (int k = 0; k < U; k++) {
+                const long long key = key_of(t[k]);
                 s[k & 1] += t[k];
-                lo = min(lo, key_of(t[k]));
-                hi = max(hi, key_of(t[k]));
+                lo = min(lo, key);
+                hi = max(hi, key);
             }
         }
 #pragma unroll 4
         for (; m < m1; m += COL_WARPS) {
             const double t = x[(size_t)m * nbin + b];
+            const long long key = key_of(t);
             s[0] += t;
-            lo = min(lo, key_of(t));
-            hi = max(hi, key_of(t));
+            lo = min(lo, key);
+            hi = max(hi, key);
         }
     }
     sh[warp][lane] = ColPartial{s[0] + s[1], lo, hi};
@@ -84,10 +85,10 @@ __global__ void __launch_bounds__(32 * COL_WARPS)
     }
 }
 
-// Mean, lower and upper bound of column b (this thread's lane) of variant v,
-// from all partials in a fixed order; called by every thread of a block of 32
-// x COL_WARPS.  The bounds are within 2^-20 of the extrema; a column with a
-// NaN has a NaN mean.
+// Mean, smallest and largest entry of column b (this thread's lane) of variant
+// v, from all partials in a fixed order; called by every thread of a block of
+// 32 x COL_WARPS.  A column with a NaN has a NaN mean (its extrema need not be
+// numbers).
 __device__ __forceinline__ void column_stats(const ColPartial *__restrict__ part, int v, int n_mock, int nbin, int b,
                                              double &mean, double &lo, double &hi)
 {
@@ -119,8 +120,8 @@ __device__ __forceinline__ void column_stats(const ColPartial *__restrict__ part
             p.hi = max(p.hi, sh[w][lane].hi);
         }
         smean[lane] = p.sum / (double)n_mock;
-        slo[lane] = key_bound(p.lo, false);
-        shi[lane] = key_bound(p.hi, true);
+        slo[lane] = of_key(p.lo);
+        shi[lane] = of_key(p.hi);
     }
     __syncthreads();
     mean = smean[lane];
