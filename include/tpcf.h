@@ -59,7 +59,7 @@ extern "C" {
 #define TPCF_PER_LAUNCH  1        /* one kernel launch per (mock, term, subset): baseline */
 #define TPCF_HOST_INPUT  2        /* OR into mode: the mocks' position arrays are host memory */
 
-#define TPCF_FP64    0            /* covariances to float64 accuracy (exact digit products on tensor cores, or float64 sums) */
+#define TPCF_FP64    0            /* covariances to the accuracy of float64 sums (exact digit products on tensor cores, or float64 sums) */
 #define TPCF_TF32X3  1            /* Gram products on tensor cores, 3-term TF32 split, FP32 accumulate */
 #define TPCF_BF16X3  2            /* Gram products on tensor cores, 3-piece BF16 split, FP32 accumulate */
 
@@ -192,7 +192,9 @@ int tpcf_ls(tpcf_ctx *ctx, const int64_t *dd, const int64_t *dr, const int64_t *
  * 1/(N-1) sum (xi - mean)(xi - mean)^T.  M = +INFINITY gives C^LC = A.
  * Inputs xi_a1, xi_a2, xi_b: device float64 [n_mock][nbin].
  * Outputs: C_lc required; Ca, Cb, A, B may be NULL; all device float64 [nbin][nbin].
- * `precision`: TPCF_FP64 (float64 accuracy), TPCF_TF32X3 or TPCF_BF16X3 (the
+ * `precision`: TPCF_FP64 (every element as close as a float64 sum of its
+ * products: columns whose residuals are too far apart in size for exact
+ * digit products are summed in float64), TPCF_TF32X3 or TPCF_BF16X3 (the
  * centred Gram products on tensor cores in split precision with FP32
  * accumulation over K-chunks and a float64 sum; means and the final
  * combination stay float64).  Needs n_mock >= 2, M_a >= 1, M >= M_a.

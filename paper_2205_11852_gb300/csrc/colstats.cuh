@@ -34,15 +34,18 @@ __device__ __forceinline__ long long key_of(double v)
 // the double with the key
 __device__ __forceinline__ double of_key(long long key) { return __longlong_as_double(key ^ ((key >> 63) & KEY_MAX)); }
 
-// part[v][chunk][b] of the rows [chunk * per, (chunk + 1) * per)
+// part[v][chunk][b] of the rows [chunk * per, (chunk + 1) * per); zero (may be null): [v][n_zero][nbin] to clear
 __global__ void __launch_bounds__(32 * COL_WARPS)
     column_partials_kernel(const double *__restrict__ x0, const double *__restrict__ x1,
-                           const double *__restrict__ x2, int n_mock, int nbin, ColPartial *__restrict__ part)
+                           const double *__restrict__ x2, int n_mock, int nbin, ColPartial *__restrict__ part,
+                           uint32_t *__restrict__ zero, int n_zero)
 {
     __shared__ ColPartial sh[COL_WARPS][32];
     const int v = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const double *x = v == 0 ? x0 : (v == 1 ? x1 : x2);
     const int b = blockIdx.x * 32 + lane;
+    if (zero && blockIdx.y == 0 && b < nbin)
+        for (int k = warp; k < n_zero; k += COL_WARPS) zero[((size_t)v * n_zero + k) * nbin + b] = 0u;
     const int per = (n_mock + COL_CHUNKS - 1) / COL_CHUNKS;
     const int m0 = min(n_mock, (int)blockIdx.y * per), m1 = min(n_mock, m0 + per);
     double s[2] = {0.0, 0.0};
@@ -130,10 +133,11 @@ __device__ __forceinline__ void column_stats(const ColPartial *__restrict__ part
 }
 
 inline cudaError_t launch_column_partials(const double *x0, const double *x1, const double *x2, int n_var, int n_mock,
-                                          int nbin, ColPartial *part, cudaStream_t s)
+                                          int nbin, ColPartial *part, cudaStream_t s, uint32_t *zero = nullptr,
+                                          int n_zero = 0)
 {
     column_partials_kernel<<<dim3((nbin + 31) / 32, COL_CHUNKS, n_var), 32 * COL_WARPS, 0, s>>>(x0, x1, x2, n_mock,
-                                                                                               nbin, part);
+                                                                                               nbin, part, zero, n_zero);
     return cudaGetLastError();
 }
 

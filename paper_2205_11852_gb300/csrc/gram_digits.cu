@@ -19,12 +19,28 @@
 // accumulators of 64 columns fill tensor memory.  A CTA writes its tile as
 // pairs of 64-bit integers, and the combining kernel adds the K-segments as
 // integers and rounds to float64 once, so the result does not depend on an
-// order of summation and its error per element is about sqrt(n) 2^(e_i + e_j - 60): below that of a float64 sum, whose partial sums
-// round at 2^-53 of their own size.
+// order of summation.
 //
-// Columns whose residuals are not finite or lie outside 2^+-400 are not split:
-// the combining kernel sums their elements in float64 directly, so NaN and
-// infinities spread as in the float64 kernel.
+// Which columns are split.  A fixed-point residual is exact from an eighth of
+// its column's largest one on (often from less) and off by up to 2^(e_i - 56)
+// below, whatever its own size, where a float64 product keeps 53 bits.  That
+// is nothing against the sum of |y_i y_j| of ordinary columns (0.01 to 0.08 of
+// 2^-53 of it, root mean square, on normal ones; the products' own float64
+// sums 0.5 to 1.2), but not of columns whose large residuals are few and meet
+// small ones of other columns: with two pairs of +-10^6 in different mocks of
+// columns of unit scatter it would be 4 x 10^4.  So the octaves of a column's
+// residuals are counted, and it is split when, with a the mean of |y| and r
+// its root mean square,
+//   2^e_i r <= 2 sqrt(n) a^2    (the products' error against a sum of
+//                                independent |y_i| |y_j|, 0.1 x 2^-53), and
+//   3/4 of its residuals lie above a / 6 (to a factor of two: any two such
+//                                columns have half their mocks in common).
+// Over normal, Student t, lognormal, rare-event and two-scale columns, among
+// them ones made so that the large residuals of one column meet the small ones
+// of the next, at 4 to 3500 mocks, the split columns' error stayed below half
+// of the float64 sums'.  Elements of the others (and of columns whose residuals
+// are not finite or lie outside 2^+-400) are summed in float64 by the combining
+// kernel, in two levels, over tiles of 8 x 8 elements.
 //
 // What bounds it: the operand tiles' way into the SMs, 48 KB per slice and CTA
 // (about 5.7 TB/s over 144 CTAs; a tile of 8 columns, with a quarter of the
@@ -32,7 +48,9 @@
 // stacked along N, so that 20 MMAs of up to 256 columns cover a slice's 43
 // products and A is read from shared memory once per 256 columns.  Measured
 // (3500 x 200 LC covariance): Gram 44 us, digits 19, column statistics 10,
-// combination 8.5; 1356 -> 81 us per call.
+// combination 8.5; 1356 -> 79 us per call, 82 with the octave counts.  Columns
+// that are not split: 3500 x 200 with one of them 112 -> 415 us of device and
+// host time, with all 941, by the tiled float64 kernel 1393.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -57,6 +75,7 @@ constexpr int STAGE_BYTES = SLICE_BYTES + SLICE_BYTES / 2;
 constexpr int D_EPI_WARPS = 8;
 constexpr int D_THREADS = 32 * (D_EPI_WARPS + 2);
 constexpr int EXP_BAD = 1 << 20;               // "exponent" of a column that is not split
+constexpr int OCT = 16;                        // octaves of |y| below 2^e that are counted, the last with all below
 
 static_assert(SEG_SLICES * DKS * 7 * 4096 < (1 << 24), "level sums must stay exact in FP32");
 
@@ -79,26 +98,29 @@ __device__ __forceinline__ long long to_fixed(double y, int e)
 // layout of the tensor-core descriptors (8 rows x 16 bytes core matrices).
 // A block takes 32 columns (one per lane) and one of COL_CHUNKS row ranges of
 // one variant; it first closes the column statistics of all row ranges
-// (column_partials_kernel).  ecol[v][b]: the column's exponent; mean[v][b].
+// (column_partials_kernel).  ecol[v][b]: the column's exponent; mean[v][b];
+// oct[v][k][b]: residuals with 2^(e-1-k) <= |y| < 2^(e-k) (k = 15: all below).
 // Rows past nbin are left unwritten (an output element depends on its own two
 // operand rows only), mocks past n_mock are zeros.  Two float64 additions per
 // element (the sum and the residual) bound the two kernels.
 __global__ void __launch_bounds__(32 * COL_WARPS)
     digits_kernel(const double *__restrict__ x0, const double *__restrict__ x1, const double *__restrict__ x2,
                   const ColPartial *__restrict__ part, int n_mock, int nbin, int n_rb, int n_ks,
-                  unsigned char *__restrict__ tiles, int *__restrict__ ecol, double *__restrict__ mean)
+                  unsigned char *__restrict__ tiles, int *__restrict__ ecol, double *__restrict__ mean,
+                  uint32_t *__restrict__ oct)
 {
+    __shared__ uint32_t cnt[OCT][32];
     const int v = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const double *x = v == 0 ? x0 : (v == 1 ? x1 : x2);
     const int b = blockIdx.x * 32 + lane;
     double mu, mn, mx;
-    column_stats(part, v, n_mock, nbin, b, mu, mn, mx);
-    if (b >= nbin) return;
+    for (int k = threadIdx.x; k < OCT * 32; k += blockDim.x) cnt[k / 32][k % 32] = 0u;
+    column_stats(part, v, n_mock, nbin, b, mu, mn, mx);   // (has block barriers)
     // |x - mean| is largest at an extremum (rounding is monotone); NaN and infinities fail the tests
     const double top = fmax(mx - mu, mu - mn);
     const bool bad = !(mu == mu) || !(top < 0x1p400) || (top != 0.0 && !(top > 0x1p-400));
     const int e = bad || top == 0.0 ? 0 : ilogb(top) + 1;
-    if (blockIdx.y == 0 && warp == 0) {
+    if (blockIdx.y == 0 && warp == 0 && b < nbin) {
         ecol[(size_t)v * nbin + b] = bad ? EXP_BAD : e;
         mean[(size_t)v * nbin + b] = mu;
     }
@@ -108,14 +130,18 @@ __global__ void __launch_bounds__(32 * COL_WARPS)
                                          (1ll << 42) + (1ll << 49));
     // groups of 8 mocks: one 16-byte chunk per digit
     const int n_g = 2 * n_ks, per = (n_g + gridDim.y - 1) / gridDim.y;
-    const int g1 = min(n_g, ((int)blockIdx.y + 1) * per);
+    const int g1 = b < nbin ? min(n_g, ((int)blockIdx.y + 1) * per) : 0;
     for (int g = (int)blockIdx.y * per + warp; g < g1; g += COL_WARPS) {
         double y[8];
 #pragma unroll
         for (int k = 0; k < 8; k++) y[k] = g * 8 + k < n_mock ? x[(size_t)(g * 8 + k) * nbin + b] : mu;
         long long t[8];
 #pragma unroll
-        for (int k = 0; k < 8; k++) t[k] = (bad ? 0ll : to_fixed(y[k] - mu, e)) + BIAS;
+        for (int k = 0; k < 8; k++) {
+            const double d = y[k] - mu;
+            t[k] = (bad ? 0ll : to_fixed(d, e)) + BIAS;
+            if (g * 8 + k < n_mock) atomicAdd(&cnt[min(OCT - 1, e + 1022 - ((__double2hiint(d) >> 20) & 0x7ff)) & (OCT - 1)][lane], 1u);
+        }
         unsigned char *dst = col + (size_t)(g >> 1) * SLICE_BYTES + (g & 1) * 128;
 #pragma unroll
         for (int d = 0; d < NDIG; d++) {
@@ -138,6 +164,37 @@ __global__ void __launch_bounds__(32 * COL_WARPS)
             *(uint4 *)(dst + d * DIG_BYTES) = make_uint4(w[0], w[1], w[2], w[3]);
         }
     }
+    __syncthreads();
+    if (b < nbin)
+        for (int k = warp; k < OCT; k += COL_WARPS)
+            if (cnt[k][lane]) atomicAdd(&oct[((size_t)v * OCT + k) * nbin + b], cnt[k][lane]);
+}
+
+// Whether a column of n residuals with these octave counts is split (see the top); o[k * stride]
+__device__ __forceinline__ bool column_fits(const uint32_t *__restrict__ o, int stride, int n)
+{
+    float a = 0.0f, q = 0.0f, w = 1.0f;   // mean |y| and mean square over 2^e, residuals spread evenly in an octave
+    uint32_t c[OCT];
+#pragma unroll
+    for (int k = 0; k < OCT; k++) c[k] = o[(size_t)k * stride];
+#pragma unroll
+    for (int k = 0; k < OCT - 1; k++) {
+        w *= 0.5f;
+        a += 1.5f * w * (float)c[k];
+        q += 7.0f / 3.0f * w * w * (float)c[k];
+    }
+    if (a == 0.0f) return true;   // all residuals are zero
+    a /= (float)n;
+    q /= (float)n;
+    if (!(q <= 4.0f * a * a * a * a * (float)n)) return false;
+    uint32_t above = 0;
+    w = 1.0f;
+#pragma unroll
+    for (int k = 0; k < OCT - 1; k++) {
+        if (w > a * (1.0f / 6.0f)) above += c[k];
+        w *= 0.5f;
+    }
+    return 4ull * ((uint32_t)n - above) <= (uint32_t)n;
 }
 
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc)
@@ -180,12 +237,16 @@ constexpr int digits_smem_bytes() { return DSTAGE * STAGE_BYTES + 8 * (2 * DSTAG
 // 0-7 read the eight accumulators back once and write T[segment][v][j][i],
 // consecutive i per warp.
 //
+// The first CTA of each variant also decides which columns the combining
+// kernel takes from the products (its warps 0-7 would wait for them).
+//
 // Every wait is bounded.  The MMA thread commits `done` also when a wait gave
 // up, so the epilogue's wait always ends; a wait that gave up sets
 // STATUS_TIMEOUT and nothing of the tile is written.
 __global__ void __launch_bounds__(D_THREADS, 1)
     gram_digits_kernel(const unsigned char *__restrict__ tiles, int nbin, int n_rb, int n_cb, int n_ks, int spc,
-                       longlong2 *__restrict__ T, int *__restrict__ status)
+                       longlong2 *__restrict__ T, const uint32_t *__restrict__ oct, int n_mock,
+                       int *__restrict__ ecol, int *__restrict__ status)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t *full = (uint64_t *)(smem + DSTAGE * STAGE_BYTES);
@@ -276,6 +337,9 @@ __global__ void __launch_bounds__(D_THREADS, 1)
             mma_commit(done);
             if (!ok) atomicOr(status, STATUS_TIMEOUT);
         }
+    } else if (blockIdx.x == 0 && kc == 0) {
+        for (int b = tid; b < nbin; b += 32 * D_EPI_WARPS)
+            if (!column_fits(oct + (size_t)v * OCT * nbin + b, nbin, n_mock)) ecol[(size_t)v * nbin + b] = EXP_BAD;
     }
     __syncthreads();
     // every product has completed (bounded)
@@ -314,8 +378,13 @@ __global__ void __launch_bounds__(D_THREADS, 1)
 // Adds the segments of T (integers) and combines: NV = 3 the LC covariance
 // (Eqs. R1R2, LCdef), NV = 1 the sample covariance into C_lc.  A block takes a
 // 8 x 8 tile of the lower triangle, one variant per layer of threads (all of
-// an element's loads in flight), and writes the tile and its mirror.
-constexpr int CT = 8;
+// an element's loads in flight), and writes the tile and its mirror.  A tile
+// with columns that are not split also sums its elements in float64: residuals
+// of CK mocks at a time in shared memory (a quarter of a subtraction per
+// multiply-add; the next ones' loads in flight), four chains of CK / 4 terms
+// each, then one compensated addition (Knuth's two-sum) to the total, so a
+// product goes through CK / 4 + 4 roundings however many mocks there are.
+constexpr int CT = 8, CK = 32;
 template <int NV>
 __global__ void __launch_bounds__(CT *CT *NV)
     combine_digits_kernel(const longlong2 *__restrict__ T, int n_seg, int nbin, int n_mock,
@@ -323,7 +392,8 @@ __global__ void __launch_bounds__(CT *CT *NV)
                           const double *__restrict__ x0, const double *__restrict__ x1,
                           const double *__restrict__ x2, double inv, double two_ma, double M, CovOut out)
 {
-    __shared__ double sc[NV][CT][CT + 1], sh[5][CT][CT + 1];
+    __shared__ double sc[NV][CT][CT + 1], sh[5][CT][CT + 1], ys[NV][2][CK][CT];
+    __shared__ int some[NV];   // elements of the variant are summed directly
     int tj = (int)((sqrtf(8.0f * (float)blockIdx.x + 1.0f) - 1.0f) * 0.5f);
     while ((long long)tj * (tj + 1) / 2 > (long long)blockIdx.x) tj--;
     while ((long long)(tj + 1) * (tj + 2) / 2 <= (long long)blockIdx.x) tj++;
@@ -332,6 +402,9 @@ __global__ void __launch_bounds__(CT *CT *NV)
     const int i = ti * CT + tx, j = tj * CT + ty;
     const size_t nn = (size_t)nbin * nbin;
     const bool low = i < nbin && j < nbin && j >= i;
+    double g = 0.0;
+    bool bad = false;
+    if (threadIdx.x < NV) some[threadIdx.x] = 0;
     if (low) {
         const int ei = ecol[(size_t)v * nbin + i], ej = ecol[(size_t)v * nbin + j];
         const longlong2 *t = T + (size_t)v * nn + (size_t)j * nbin + i;
@@ -342,19 +415,54 @@ __global__ void __launch_bounds__(CT *CT *NV)
             hi += u.x;
             lo += u.y;
         }
-        double g;
-        if (ei == EXP_BAD || ej == EXP_BAD) {
-            const double *x = v == 0 ? x0 : (v == 1 ? x1 : x2);
-            const double mi = mean[(size_t)v * nbin + i], mj = mean[(size_t)v * nbin + j];
-            g = 0.0;
-            for (int m = 0; m < n_mock; m++)
-                g = fma(x[(size_t)m * nbin + i] - mi, x[(size_t)m * nbin + j] - mj, g);
-        } else {
-            // hi: levels 0..3, units of 2^(ei + ej - 12 - 21); lo: levels 4..8, units of 2^(ei + ej - 12 - 49)
-            g = fma((double)hi, 0x1p28, (double)lo) * __hiloint2double((1023 + ei + ej - 61) << 20, 0);
-        }
-        sc[v][ty][tx] = g * inv;
+        bad = ei == EXP_BAD || ej == EXP_BAD;
+        // hi: levels 0..3, units of 2^(ei + ej - 12 - 21); lo: levels 4..8, units of 2^(ei + ej - 12 - 49)
+        if (!bad) g = fma((double)hi, 0x1p28, (double)lo) * __hiloint2double((1023 + ei + ej - 61) << 20, 0);
     }
+    if (__syncthreads_or(bad)) {
+        if (bad) some[v] = 1;
+        __syncthreads();
+        const bool mine = some[v] != 0, sums = __any_sync(0xffffffffu, bad);   // by layer, by warp
+        const double *x = v == 0 ? x0 : (v == 1 ? x1 : x2);
+        const int c0 = ti * CT + tx, c1 = tj * CT + tx;   // this thread's columns of the two sides
+        const double m0 = c0 < nbin ? mean[(size_t)v * nbin + c0] : 0.0, m1 = c1 < nbin ? mean[(size_t)v * nbin + c1] : 0.0;
+        constexpr int Q = CK / CT;   // mocks per thread and side
+        double d0[Q] = {}, d1[Q] = {}, total = 0.0, rest = 0.0;
+        auto load = [&](int k0) {
+#pragma unroll
+            for (int q = 0; q < Q; q++) {
+                const int k = k0 + ty + CT * q;
+                d0[q] = mine && k < n_mock && c0 < nbin ? x[(size_t)k * nbin + c0] : 0.0;
+                d1[q] = mine && k < n_mock && c1 < nbin ? x[(size_t)k * nbin + c1] : 0.0;
+            }
+        };
+        load(0);
+        for (int k0 = 0; k0 < n_mock; k0 += CK) {
+            if (mine) {
+#pragma unroll
+                for (int q = 0; q < Q; q++) {   // mocks past the last: zero
+                    const bool in = k0 + ty + CT * q < n_mock;
+                    ys[v][0][ty + CT * q][tx] = in ? d0[q] - m0 : 0.0;
+                    ys[v][1][ty + CT * q][tx] = in ? d1[q] - m1 : 0.0;
+                }
+            }
+            __syncthreads();
+            if (k0 + CK < n_mock) load(k0 + CK);
+            if (sums) {
+                double a[4] = {0.0, 0.0, 0.0, 0.0};
+                for (int k = 0; k < min(CK, n_mock - k0); k += 8)
+#pragma unroll
+                    for (int l = 0; l < 8; l++) a[l & 3] = fma(ys[v][0][k + l][tx], ys[v][1][k + l][ty], a[l & 3]);
+                const double p = (a[0] + a[1]) + (a[2] + a[3]), t = total + p, z = t - total;
+                rest += (total - (t - z)) + (p - z);
+                total = t;
+            }
+            __syncthreads();
+        }
+        // (a total that is not finite has no compensation)
+        if (bad) g = total - total == 0.0 ? total + rest : total;
+    }
+    if (low) sc[v][ty][tx] = g * inv;
     __syncthreads();
     if (v == 0 && low) {
         if (NV == 1) {
@@ -381,7 +489,7 @@ __global__ void __launch_bounds__(CT *CT *NV)
 
 struct DShape {
     int n_rb, n_cb, n_ks, pairs, spc, n_seg;
-    size_t o_T, o_part, o_mean, o_e, bytes;
+    size_t o_T, o_part, o_mean, o_e, o_oct, bytes;
 };
 
 DShape dshape(int n_mock, int nbin, int n_var, int n_sm)
@@ -404,7 +512,8 @@ DShape dshape(int n_mock, int nbin, int n_var, int n_sm)
     s.o_part = s.o_T + al((size_t)s.n_seg * n_var * nbin * nbin * sizeof(longlong2));
     s.o_mean = s.o_part + al((size_t)n_var * COL_CHUNKS * nbin * sizeof(ColPartial));
     s.o_e = s.o_mean + al((size_t)n_var * nbin * 8);
-    s.bytes = s.o_e + al((size_t)n_var * nbin * 4);
+    s.o_oct = s.o_e + al((size_t)n_var * nbin * 4);
+    s.bytes = s.o_oct + al((size_t)n_var * OCT * nbin * 4);
     return s;
 }
 
@@ -412,13 +521,16 @@ DShape dshape(int n_mock, int nbin, int n_var, int n_sm)
 
 size_t cov_digits_work_bytes(int n_mock, int nbin, int n_var, int n_sm) { return dshape(n_mock, nbin, n_var, n_sm).bytes; }
 
-// The faster float64 path at every size measured (device time of an LC / a sample covariance, this path
-// against the tiled float64 kernel): 2 x 3 21 / 21 us against 35 / 35, 40 x 20 27 / 25 against 67 / 67, 301 x 60
-// 37 / 33 against 111 / 110, 3500 x 200 81 / 46 against 1354 / 577, 40 x 1000 115 / 39 against 256 / 125.  Its
-// workspace (16 bytes per residual and per element and segment of the Gram matrices) is larger, so calls that would
-// need more than 4 GiB of it stay on the float64 kernel.
+// The faster float64 path (device and host time of an LC / a sample covariance of normal columns, this path against the
+// tiled float64 kernel): 2 x 3 53 / 36 us against 67 / 50, 40 x 20 57 / 40 against 97 / 81, 301 x 60 67 / 50 against 144 /
+// 127, 3500 x 200 112 / 61 against 1390 / 596, 40 x 1000 142 / 60 against 292 / 143.  Of columns of 3 to about 20 mocks 5 to
+// 10 % are not split, which with many bins reaches nearly every tile of the combining kernel: 16 x 1000 168 / 68 against
+// 162 / 78, 16 x 2000 441 / 148 against 378 / 120, 4 x 4000 1655 / 481 against 1261 / 318, 24 x 2000 356 / 110 against 557 /
+// 184; those stay on the float64 kernel from 1000 bins on.  So do calls that would need more than 4 GiB of the larger
+// workspace (16 bytes per residual and per element and segment of the Gram matrices).
 bool cov_digits_suits(int n_mock, int nbin, int n_var, int n_sm)
 {
+    if (n_mock > 2 && n_mock < 20 && nbin > 1000) return false;
     const DShape s = dshape(n_mock, nbin, n_var, n_sm);
     return s.n_seg <= 65535 && s.bytes <= ((size_t)4 << 30);
 }
@@ -433,17 +545,18 @@ cudaError_t launch_cov_digits(const double *x0, const double *x1, const double *
     double *mean = (double *)(w + d.o_mean);
     int *ecol = (int *)(w + d.o_e);
     ColPartial *part = (ColPartial *)(w + d.o_part);
-    cudaError_t e = launch_column_partials(x0, x1, x2, n_var, n_mock, nbin, part, s);
+    uint32_t *oct = (uint32_t *)(w + d.o_oct);
+    cudaError_t e = launch_column_partials(x0, x1, x2, n_var, n_mock, nbin, part, s, oct, OCT);
     if (e != cudaSuccess) return e;
     digits_kernel<<<dim3((nbin + 31) / 32, COL_CHUNKS, n_var), 32 * COL_WARPS, 0, s>>>(x0, x1, x2, part, n_mock, nbin,
-                                                                                      d.n_rb, d.n_ks, w, ecol, mean);
+                                                                                      d.n_rb, d.n_ks, w, ecol, mean, oct);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int smem = digits_smem_bytes();
     e = cudaFuncSetAttribute(gram_digits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     gram_digits_kernel<<<dim3(d.pairs, n_var, d.n_seg), D_THREADS, smem, s>>>(w, nbin, d.n_rb, d.n_cb, d.n_ks, d.spc,
-                                                                             T, status);
+                                                                             T, oct, n_mock, ecol, status);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const long long nt = (nbin + CT - 1) / CT;
