@@ -379,13 +379,12 @@ __global__ void __launch_bounds__(32 * TS_WARPS)
 // that its norm lies in [1, 2): the number of sign changes is the number of
 // eigenvalues below x, without a division per step, and each step rounds like
 // the ratio form of the Sturm sequence, so the count is that of a matrix
-// within a few ulps of T.  t[i] = (d_i, e2_{i-1}), e2 at least 2^-180 (a
-// perturbation of T by 2^-90).  An exact zero becomes a tiny value of the
-// opposite sign of p_{i-1}, which no later comparison can tell from it.  The
-// pair (p_i, p_{i-1}) is rescaled by a power of two (exactly) every four
-// steps: its larger member changes by 2^-183 to 2^3 per step, so it stays
-// within 2^+-950 in between.  Returns the count; (m, ex): the last continuant
-// as m 2^ex.
+// within a few ulps of T.  t[i] = (d_i, e2_{i-1}), e2 at least 2^-180.  An
+// exact zero becomes a tiny value of the opposite sign of p_{i-1}, which no
+// later comparison can tell from it.  The pair (p_i, p_{i-1}) is rescaled by a
+// power of two (exactly) every four steps: its larger member changes by 2^-183
+// to 2^3 per step, so it stays within 2^+-950 in between.  Returns the count;
+// (m, ex): the last continuant as m 2^ex.
 __device__ __forceinline__ int sturm_count(const double2 *t, int n, double x, double &m, int &ex)
 {
     double pm = 0.0, p = 1.0;
@@ -418,6 +417,33 @@ __device__ __forceinline__ int sturm_count(const double2 *t, int n, double x, do
         }
     }
     for (; i < n; i++) step(t[i]);
+    m = p;
+    ex = shift;
+    return c;
+}
+
+// The same for a T with smaller off-diagonals, down to exact zeros (a diagonal
+// matrix, blocks that do not couple): p_i alone may fall by any factor in a
+// step, so the pair is rescaled whenever p_i leaves [2^-300, 2^300], and an
+// exact zero becomes -2^-400 p_{i-1}.
+__device__ __noinline__ int sturm_count_apart(const double2 *t, int n, double x, double &m, int &ex)
+{
+    double pm = 0.0, p = 1.0;
+    int c = 0, shift = 0;
+#pragma unroll 1
+    for (int i = 0; i < n; i++) {
+        double pn = fma(t[i].x - x, p, -(t[i].y * pm));
+        if (pn == 0.0) pn = -0x1p-400 * p;
+        c += (int)((uint32_t)(__double2hiint(pn) ^ __double2hiint(p)) >> 31);
+        pm = p;
+        p = pn;
+        const int eb = (__double2hiint(p) >> 20) & 0x7ff;
+        if (eb > 1023 + 300 || eb < 1023 - 300) {
+            p = scalbn(p, 1023 - eb);
+            pm = scalbn(pm, 1023 - eb);
+            shift += eb - 1023;
+        }
+    }
     m = p;
     ex = shift;
     return c;
@@ -463,10 +489,13 @@ __global__ void __launch_bounds__(32) multisect_kernel(const double *__restrict_
         return;
     }
     const int ks = ilogb(nrm);   // T / 2^ks has its norm in [1, 2)
+    bool small = false;
     for (int k = lane; k < n; k += 32) {
         const double ek = k > 0 ? scalbn(e[k - 1], -ks) : 0.0;
-        st[k] = make_double2(scalbn(d[k], -ks), k > 0 ? fmax(ek * ek, 0x1p-180) : 0.0);
+        st[k] = make_double2(scalbn(d[k], -ks), ek * ek);
+        small |= k > 0 && ek * ek < 0x1p-180;
     }
+    const bool apart = __any_sync(0xffffffffu, small);
     __syncwarp();
     const double pad = 4e-16 * n;
     lo = scalbn(lo, -ks) - pad;
@@ -500,7 +529,7 @@ __global__ void __launch_bounds__(32) multisect_kernel(const double *__restrict_
         const double x = fma(h, (double)frac, lo);
         double m;
         int ex;
-        const int c = sturm_count(st, n, x, m, ex);
+        const int c = apart ? sturm_count_apart(st, n, x, m, ex) : sturm_count(st, n, x, m, ex);
         const bool above = c > i;
         // the highest point that is not above and the lowest that is (lane 31's point takes part in neither)
         const long long kx = key(x), none = 0x7fffffffffffffffll;
