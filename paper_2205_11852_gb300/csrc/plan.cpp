@@ -572,15 +572,19 @@ bool build_direct(const tpcf_binning &b, const Plan &pl, int smem_sm, int smem_b
         if ((op.R == 32 && d.logC > 5) || (op.R == 8 && d.logC < 5)) continue;
         const long long need = (long long)pairdirect_smem_bytes(p, d.rows, op.R, d.C, op.NT, W);
         if (need > budget) continue;
+        // in one unit a lane pairs at most 64 a-points with at most
+        // max_cat / 32 + 16 b-points (its tile slots), and 32 / R
+        // lanes share a counter copy; a unit that could wrap a 32-bit counter
+        // by itself (one copy, catalogues above 67 million points) leaves the
+        // call to the general counter
+        const unsigned long long bound = (unsigned long long)DIRECT_ACHUNK * (max_cat / (unsigned long long)op.R +
+                                                                              512ull / (unsigned long long)op.R + 16ull);
+        if (bound > 0xFFFFFFFFull) continue;
         d.NT = op.NT;
         d.R = op.R;
         d.W = W;
         d.smem = (int)need;
-        // in one unit a lane pairs at most 64 a-points with at most
-        // max_cat / 32 + 16 b-points (its tile slots), and 32 / R
-        // lanes share a counter copy
-        d.unit_pair_bound = (unsigned long long)DIRECT_ACHUNK * (max_cat / (unsigned long long)op.R +
-                                                                 512ull / (unsigned long long)op.R + 16ull);
+        d.unit_pair_bound = bound;
         return true;
     }
     return false;
