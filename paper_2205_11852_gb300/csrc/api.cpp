@@ -223,6 +223,7 @@ int tpcf_create(tpcf_ctx **out, int cuda_device)
     }
     if (const char *v = std::getenv("TPCF_TEST_FAIL_ALLOC")) ctx->fail_alloc_at = std::atoll(v);
     if (const char *v = std::getenv("TPCF_TEST_FAIL_COUNT")) ctx->fail_count_at = std::atoll(v);
+    if (const char *v = std::getenv("TPCF_TEST_MAX_CLUSTER")) ctx->test_max_cluster = std::atoi(v);
     *out = ctx;
     return TPCF_OK;
 }
@@ -564,7 +565,7 @@ int tpcf_eigvalsh(tpcf_ctx *ctx, const double *C, int n, double *w, void *stream
     if (n < 1 || n > 1024) return fail(ctx, TPCF_ERR_ARG, "eigenvalues need 1 <= n <= 1024");
     void *wk;
     if ((rc = ensure(ctx, "eig_work", eig_work_bytes(n), &wk))) return rc;
-    CK(launch_eigvalsh(C, n, (double *)wk, w, (cudaStream_t)stream));
+    CK(launch_eigvalsh(C, n, (double *)wk, w, ctx->test_max_cluster, (cudaStream_t)stream));
     return TPCF_OK;
 }
 

@@ -563,39 +563,63 @@ __global__ void __launch_bounds__(32) multisect_kernel(const double *__restrict_
 
 int blocks_for(size_t n, int threads) { return (int)std::max<size_t>(1, std::min<size_t>((n + threads - 1) / threads, 152 * 16)); }
 
+// Launch shape of the shared-memory reduction in a cluster of C blocks
+template <int C>
+struct ClusterLaunch {
+    cudaLaunchAttribute at[1];
+    cudaLaunchConfig_t cfg = {};
+    ClusterLaunch(int n, cudaStream_t s)
+    {
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = C;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(C);
+        cfg.blockDim = dim3(32 * TS_WARPS);
+        cfg.dynamicSmemBytes = tri_smem_bytes(n, C);
+        cfg.stream = s;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+    }
+    ClusterLaunch(const ClusterLaunch &) = delete;
+};
+
+// The matrix fits in the shared memory of C blocks and the device runs clusters of that size and footprint (more than 8
+// blocks is not guaranteed: a partition may hold fewer SMs of one cluster's reach).  max_cluster > 0 (tests) stands in
+// for the device's answer.
+template <int C>
+bool cluster_fits(int n, int max_cluster)
+{
+    constexpr size_t room = (size_t)226 << 10;
+    ClusterLaunch<C> l(n, nullptr);
+    const size_t sb = l.cfg.dynamicSmemBytes;
+    if (sb > room || (max_cluster > 0 && C > max_cluster)) return false;
+    int held = 0;
+    bool ok = cudaFuncSetAttribute(tridiag_smem_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb) == cudaSuccess;
+    if (ok && C > 8)
+        ok = cudaFuncSetAttribute(tridiag_smem_kernel<C>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    ok = ok && cudaOccupancyMaxActiveClusters(&held, tridiag_smem_kernel<C>, &l.cfg) == cudaSuccess && held > 0;
+    if (!ok) cudaGetLastError();
+    return ok;
+}
+
 template <int C>
 cudaError_t launch_tridiag_smem(const double *A, int n, double *d, double *e, cudaStream_t s)
 {
-    const size_t sb = tri_smem_bytes(n, C);
-    cudaError_t err = cudaFuncSetAttribute(tridiag_smem_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb);
-    if (err == cudaSuccess && C > 8)
-        err = cudaFuncSetAttribute(tridiag_smem_kernel<C>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (err != cudaSuccess) return err;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = C;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(C);
-    cfg.blockDim = dim3(32 * TS_WARPS);
-    cfg.dynamicSmemBytes = sb;
-    cfg.stream = s;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, tridiag_smem_kernel<C>, A, n, d, e);
+    ClusterLaunch<C> l(n, s);
+    return cudaLaunchKernelEx(&l.cfg, tridiag_smem_kernel<C>, A, n, d, e);
 }
 
 // The cluster size of the shared-memory reduction for order n: 16 blocks (an
-// opt-in size) from n = 96, below which 8 do as well, else 8; 0 when the matrix
-// does not fit (n > 628).  Whole call with 16 / with 8 / before: n = 96
+// opt-in size) from n = 96, below which 8 do as well, else 8; 0 when neither
+// holds the matrix (n > 628) or the device has no room for such a cluster.
+// Whole call with 16 / with 8 / before: n = 96
 // 497 / 497 / 874 us, 120 675 / 698 / 1134, 200 1224 / 1434 / 2125, 420 4132 /
 // 5930 / 6794, 600 8458 / - / 16750.
-int pick_cluster(int n)
+int pick_cluster(int n, int max_cluster)
 {
-    constexpr size_t room = (size_t)226 << 10;
-    if (n >= 96 && tri_smem_bytes(n, 16) <= room) return 16;
-    return tri_smem_bytes(n, 8) <= room ? 8 : 0;
+    if (n >= 96 && cluster_fits<16>(n, max_cluster)) return 16;
+    return cluster_fits<8>(n, max_cluster) ? 8 : 0;
 }
 
 }  // namespace
@@ -628,12 +652,12 @@ cudaError_t launch_chi2(int mode, const double *X, const double *Y, const double
 
 size_t eig_work_bytes(int n) { return ((size_t)n * n + 3 * (size_t)n) * sizeof(double); }
 
-cudaError_t launch_eigvalsh(const double *C, int n, double *work, double *w, cudaStream_t s)
+cudaError_t launch_eigvalsh(const double *C, int n, double *work, double *w, int max_cluster, cudaStream_t s)
 {
     double *a = work, *d = work + (size_t)n * n, *e = d + n, *pg = e + n;
     cudaError_t err;
-    int cl = 0;   // blocks of the cluster whose shared memory holds the matrix; 0: it does not fit
-    if (n >= 3) cl = pick_cluster(n);
+    int cl = 0;   // blocks of the cluster whose shared memory holds the matrix; 0: none does
+    if (n >= 3) cl = pick_cluster(n, max_cluster);
     if (cl == 16) {
         err = launch_tridiag_smem<16>(C, n, d, e, s);
         if (err != cudaSuccess) return err;

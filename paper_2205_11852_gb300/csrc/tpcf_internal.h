@@ -238,6 +238,7 @@ cudaError_t launch_chi2(int mode, const double *X, const double *Y, const double
                         double *work, double *out, cudaStream_t s);
 size_t eig_work_bytes(int n);
 // ascending eigenvalues w[n] of the symmetric C[n][n] (n <= 1024)
-cudaError_t launch_eigvalsh(const double *C, int n, double *work, double *w, cudaStream_t s);
+// max_cluster > 0 (tests): the largest cluster the device is taken to hold
+cudaError_t launch_eigvalsh(const double *C, int n, double *work, double *w, int max_cluster, cudaStream_t s);
 
 }  // namespace tpcf
