@@ -1301,6 +1301,7 @@ __device__ __forceinline__ int switch_table(const CountParams &prm, const Direct
             }
         }
         if (__shfl_sync(0xffffffffu, last, 0)) {
+            __syncwarp();   // lane 0's lock came after the other warps' adds; the lanes that read the table come after it
             unsigned long long bn = drain<MU, R, LOGC>(prm, dp, terms, (uint32_t *)(tables + (size_t)tab * hstride),
                                                        hstride / 4u, wm.st->term, lane);
 #pragma unroll
@@ -1352,7 +1353,9 @@ __device__ __forceinline__ int switch_table(const CountParams &prm, const Direct
         wm.st->t_lo = t_lo;
         wm.st->t_hi = t_hi;
     }
-    return __shfl_sync(0xffffffffu, k, 0);
+    k = __shfl_sync(0xffffffffu, k, 0);
+    __syncwarp();   // the lanes' adds come after lane 0's lock, and so after the last drain's clearing
+    return k;
 }
 
 // The same as a call of its own (midpoint line of sight, see recheck_apart).
