@@ -95,7 +95,8 @@ struct Sched {
     unsigned long long claim;   // the block's claim: next unit (low word; may pass the end) and end (high word)
     unsigned n_used[MAX_NT];    // units taken for a table since it was last empty
     unsigned lock;
-    unsigned done;              // no unit is left to claim
+    unsigned short done;        // no unit is left to claim
+    unsigned short moves;       // times a table was entered or freed (modulo 2^16)
     int term[MAX_NT];           // the term a table counts, or FREE, or DRAINING
     unsigned ref[MAX_NT];       // warps adding to a table
 };
@@ -1236,7 +1237,7 @@ __device__ __forceinline__ unsigned claim_more(Sched &q, unsigned *claim, uint32
     // without the flag each warp in turn would read the used-up counter under the lock, 16 latencies of global
     // memory at the end of every launch: one launch per term of 16 mocks of 4000 points 3.66 -> 3.33 ms for the
     // whole step, batched 0.66 -> 0.64
-    if (*(volatile unsigned *)&q.done) return u;
+    if (*(volatile unsigned short *)&q.done) return u;
     if (!sched_lock(q)) {
         atomicOr(status, STATUS_TIMEOUT);
         return u;
@@ -1244,7 +1245,7 @@ __device__ __forceinline__ unsigned claim_more(Sched &q, unsigned *claim, uint32
     const unsigned long long c = atomicAdd(&q.claim, 1ull);
     if ((uint32_t)c < (uint32_t)(c >> 32)) {
         u = (uint32_t)c;
-    } else if (!*(volatile unsigned *)&q.done) {
+    } else if (!*(volatile unsigned short *)&q.done) {
         const uint32_t g = *(volatile unsigned *)claim;
         const uint32_t rem = g < span ? span - g : 0u;
         const uint32_t cmin = min(csize, max(csize / 32u, (uint32_t)DIRECT_WARPS));
@@ -1255,7 +1256,7 @@ __device__ __forceinline__ unsigned claim_more(Sched &q, unsigned *claim, uint32
             atomicExch(&q.claim,
                        (unsigned long long)(u + 1u) | (unsigned long long)(u_lo + min(span, c0 + sz)) << 32);
         } else {
-            *(volatile unsigned *)&q.done = 1u;
+            *(volatile unsigned short *)&q.done = 1;
         }
     }
     sched_unlock(q);
@@ -1268,6 +1269,63 @@ __device__ __forceinline__ unsigned most_units(const DirectParams &dp)
 {
     return (unsigned)min(0x7fffffffull, ((1ull << 32) - 1ull) / dp.unit_pair_bound);
 }
+
+// One lane finds a table for term t: the one that counts it, or a free one.
+// Returns its number, -1 when the wait gave up.
+__device__ __forceinline__ int enter_table(Sched &q, const DirectParams &dp, int t)
+{
+    int k = -1;
+    const unsigned most = most_units(dp);
+    // A table becomes free when the last of its warps leaves it.  Meanwhile
+    // they may take further units of its term, and where there is one table
+    // another term's warps may enter it first, so the wait can be long; but
+    // every such step takes a unit or moves a table, and between two steps
+    // lies at most one unit: at most R unit_pair_bound pairs, 0.1 us each
+    // when all are rechecked.  The wait gives up when nothing has happened
+    // for that long.
+    const unsigned long long limit = 4000000000ull + 100ull * (unsigned)dp.R * dp.unit_pair_bound;
+    unsigned long long since = gtimer(), seen = 0ull;
+#pragma unroll 1
+    for (;;) {
+        if (!sched_lock(q)) break;
+        unsigned long long now = 0ull;
+#pragma unroll 1
+        for (int j = 0; j < dp.NT; j++) {
+            // a full table is not counted on: its counter could wrap
+            if (k < 0 && q.term[j] == t && *(volatile unsigned *)&q.n_used[j] < most &&
+                atomicAdd(&q.n_used[j], 1u) < most)
+                k = j;
+            now += *(volatile unsigned *)&q.n_used[j];
+        }
+        now |= (unsigned long long)q.moves << 40;
+        if (k >= 0) {
+            q.ref[k]++;
+        } else {
+#pragma unroll 1
+            for (int j = 0; j < dp.NT; j++)
+                if (k < 0 && q.term[j] == FREE) k = j;
+            if (k >= 0) {
+                q.term[k] = t;
+                q.ref[k] = 1u;
+                atomicExch(&q.n_used[k], 1u);
+            }
+        }
+        if (k >= 0) q.moves++;
+        sched_unlock(q);
+        if (k >= 0) break;
+        if (now != seen) {
+            seen = now;
+            since = gtimer();
+        } else if (gtimer() - since >= limit) {
+            break;
+        }
+        __nanosleep(200);
+    }
+    return k;
+}
+
+// The same as a call of its own, see below.
+__device__ __noinline__ int enter_table_apart(Sched &q, const DirectParams &dp, int t) { return enter_table(q, dp, t); }
 
 // The warp (all lanes) leaves its table, if it has one, draining it when it is
 // the last to leave, and, if u is a unit, enters the table of u's term: the one
@@ -1310,6 +1368,7 @@ __device__ __forceinline__ int switch_table(const CountParams &prm, const Direct
                 wm.st->binned += bn;
                 if (sched_lock(q)) {
                     q.term[tab] = FREE;
+                    q.moves++;
                     sched_unlock(q);
                 } else {
                     atomicOr(status, STATUS_TIMEOUT);
@@ -1321,32 +1380,8 @@ __device__ __forceinline__ int switch_table(const CountParams &prm, const Direct
     if (u != NO_UNIT && lane == 0) {
         const int t = units[u].term;
         const uint32_t t_lo = ustart[(size_t)t * dp.n_groups], t_hi = ustart[(size_t)(t + 1) * dp.n_groups];
-        const unsigned most = most_units(dp);
-        // a table becomes free when its last warp's unit ends: at most R
-        // unit_pair_bound pairs, 0.1 us each when all are rechecked
-        const unsigned long long limit = 4000000000ull + 100ull * R * dp.unit_pair_bound, since = gtimer();
-#pragma unroll 1
-        while (k < 0 && gtimer() - since < limit) {
-            if (!sched_lock(q)) break;
-#pragma unroll 1
-            for (int j = 0; j < dp.NT; j++)   // a full table is not counted on: its counter could wrap
-                if (q.term[j] == t && *(volatile unsigned *)&q.n_used[j] < most && atomicAdd(&q.n_used[j], 1u) < most)
-                    k = j;
-            if (k >= 0) {
-                q.ref[k]++;
-            } else {
-#pragma unroll 1
-                for (int j = 0; j < dp.NT; j++)
-                    if (k < 0 && q.term[j] == FREE) k = j;
-                if (k >= 0) {
-                    q.term[k] = t;
-                    q.ref[k] = 1u;
-                    atomicExch(&q.n_used[k], 1u);
-                }
-            }
-            sched_unlock(q);
-            if (k < 0) __nanosleep(200);
-        }
+        // (inlined it costs linear bins 0.6 to 1.5 %, as a call geometric ones 3 %)
+        k = is_geo(V) ? enter_table(q, dp, t) : enter_table_apart(q, dp, t);
         if (k < 0) atomicOr(status, STATUS_TIMEOUT);
         wm.st->tab = k;
         wm.st->term = t;
@@ -1390,7 +1425,8 @@ __global__ void __launch_bounds__(W * 32, 1)
     for (int i = tid; i <= prm.n_s; i += blockDim.x) Tsh[i] = prm.T[i];
     if (tid == 0) {
         q.claim = 0ull;
-        q.lock = q.done = 0u;
+        q.lock = 0u;
+        q.done = q.moves = 0;
         for (int k = 0; k < MAX_NT; k++) {
             q.term[k] = FREE;
             q.ref[k] = q.n_used[k] = 0u;
