@@ -1156,8 +1156,9 @@ __device__ __forceinline__ void unit(const CountParams &prm, const DirectParams 
     }
 }
 
-// one warp drains a table into term t's int64 histogram and clears it
-template <bool MU, int R, int LOGC>
+// Drains a table into term t's int64 histogram and clears its hwords words: one warp, or (BLOCK) all threads of the
+// block, which clear nothing
+template <bool MU, int R, int LOGC, bool BLOCK>
 __device__ __forceinline__ unsigned long long drain(const CountParams &prm, const DirectParams &dp,
                                                     const Term *terms, uint32_t *hist, uint32_t hwords, int t,
                                                     int lane)
@@ -1166,7 +1167,7 @@ __device__ __forceinline__ unsigned long long drain(const CountParams &prm, cons
     const int n_mu = prm.n_mu;
     unsigned long long binned = 0;
 #pragma unroll 1
-    for (int b = lane; b < prm.nbin; b += 32) {
+    for (int b = BLOCK ? (int)threadIdx.x : lane; b < prm.nbin; b += BLOCK ? (int)blockDim.x : 32) {
         const int k = b / n_mu + dp.row0, j = b % n_mu;
         unsigned long long sum = 0;
         if (R == 1) {   // one copy, one column per |mu| bin
@@ -1194,6 +1195,7 @@ __device__ __forceinline__ unsigned long long drain(const CountParams &prm, cons
         if (sum) atomicAdd((unsigned long long *)&th[b], sum);
         binned += sum;
     }
+    if (BLOCK) return binned;
     __syncwarp();
 #pragma unroll 1
     for (uint32_t i = (uint32_t)lane; i < hwords / 4; i += 32) ((uint4 *)hist)[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -1223,15 +1225,23 @@ __device__ __forceinline__ void sched_unlock(Sched &q)
 
 constexpr unsigned NO_UNIT = 0xFFFFFFFFu;
 
+// Smallest claim: csize / 32 units, or one per warp
+__device__ __forceinline__ uint32_t least_claim(uint32_t csize)
+{
+    return min(csize, max(csize / 32u, (uint32_t)DIRECT_WARPS));
+}
+
 // The block's claim is used up: one lane takes the next unit of the claim
 // that another warp made meanwhile, or makes a new one.  Claims shrink toward
 // the end (guided self-scheduling): a block takes half of the remaining units'
-// fair share, at most csize units and at least csize / 32 or one per warp, so
-// the last claims, which set the launch's tail, are short.  A stale read of
-// the counter only changes a claim's length; the atomic add keeps the claims
-// disjoint and covering.
-__device__ __forceinline__ unsigned claim_more(Sched &q, unsigned *claim, uint32_t u_lo, uint32_t span, uint32_t csize,
-                                            int *status)
+// fair share, at most csize units and at least least_claim(), so the last
+// claims, which set the launch's tail, are short.  The first `base` units are
+// not on the counter (the blocks' first claims in a launch of one term).  A
+// stale read of the counter only changes a claim's length; the atomic add
+// keeps the claims disjoint and covering.
+template <bool ONE>
+__device__ __forceinline__ unsigned claim_more(Sched &q, unsigned *claim, uint32_t u_lo, uint32_t base, uint32_t span,
+                                            uint32_t csize, int *status)
 {
     unsigned u = NO_UNIT;
     // without the flag each warp in turn would read the used-up counter under the lock, 16 latencies of global
@@ -1246,11 +1256,10 @@ __device__ __forceinline__ unsigned claim_more(Sched &q, unsigned *claim, uint32
     if ((uint32_t)c < (uint32_t)(c >> 32)) {
         u = (uint32_t)c;
     } else if (!*(volatile unsigned short *)&q.done) {
-        const uint32_t g = *(volatile unsigned *)claim;
+        const uint32_t g = *(volatile unsigned *)claim + (ONE ? base : 0u);
         const uint32_t rem = g < span ? span - g : 0u;
-        const uint32_t cmin = min(csize, max(csize / 32u, (uint32_t)DIRECT_WARPS));
-        const uint32_t sz = max(cmin, min(csize, rem / (2u * gridDim.x)));
-        const uint32_t c0 = rem ? atomicAdd(claim, sz) : span;
+        const uint32_t sz = max(least_claim(csize), min(csize, rem / (2u * gridDim.x)));
+        const uint32_t c0 = rem ? atomicAdd(claim, sz) + (ONE ? base : 0u) : span;
         if (c0 < span) {
             u = u_lo + c0;
             atomicExch(&q.claim,
@@ -1360,7 +1369,7 @@ __device__ __forceinline__ int switch_table(const CountParams &prm, const Direct
         }
         if (__shfl_sync(0xffffffffu, last, 0)) {
             __syncwarp();   // lane 0's lock came after the other warps' adds; the lanes that read the table come after it
-            unsigned long long bn = drain<MU, R, LOGC>(prm, dp, terms, (uint32_t *)(tables + (size_t)tab * hstride),
+            unsigned long long bn = drain<MU, R, LOGC, false>(prm, dp, terms, (uint32_t *)(tables + (size_t)tab * hstride),
                                                        hstride / 4u, wm.st->term, lane);
 #pragma unroll
             for (int s2 = 16; s2 > 0; s2 >>= 1) bn += __shfl_down_sync(0xffffffffu, bn, s2);
@@ -1405,7 +1414,8 @@ __device__ __noinline__ int switch_table_apart(const CountParams &prm, const Dir
                                     hb, u, n_list, status);
 }
 
-template <int V, int R, int W, int LOGC>
+// ONE: one launch per term, term_only; else all units, term_only -1.
+template <int V, int R, int W, int LOGC, bool ONE>
 __global__ void __launch_bounds__(W * 32, 1)
     pairdirect_kernel(const __grid_constant__ CountParams prm, const __grid_constant__ DirectParams dp, const Mesh m,
                       const Term *__restrict__ terms, const Unit *__restrict__ units,
@@ -1455,17 +1465,42 @@ __global__ void __launch_bounds__(W * 32, 1)
     // and units short.  Units of a few points (four per cell) suffer, since
     // warps at different places of the code share less of the instruction
     // cache (0.32 -> 0.42 ms on 16 mocks of 4000 points); the tuner takes larger
-    // cells there (0.24 ms).  With term_only >= 0 (one launch per term) only
-    // that term's units are claimed.
+    // cells there (0.24 ms).
     const uint32_t n_all = *n_units_p;
     uint32_t u_lo = 0, u_hi = n_all;
-    if (term_only >= 0) {
+    if (ONE || term_only >= 0) {   // (batched: never; without the test the batched kernels come out 0.5 to 1.3 % slower)
         u_lo = ustart[(size_t)term_only * dp.n_groups];
         u_hi = ustart[(size_t)(term_only + 1) * dp.n_groups];
     }
     const uint32_t span = u_hi - u_lo;
     const unsigned most = most_units(dp);
     Addr<MU, R, LOGC> ad{0u};
+    // One launch per term: a block's first claim is its by number (of the size
+    // the counter would give), and its warps start in the term's table and leave
+    // it together, unless the term is long enough to fill it.  Small terms'
+    // launches are too short for 16 warps to pass the lock and the counter one
+    // after another: 16 mocks of 4000 points, whole step, 3.33 -> 2.34 ms; one
+    // mock and 50 subsets of 50 000 points 28.9 -> 27.1.  Kernels of their own,
+    // since the branches cost batched launches 1 %; first claims by number cost
+    // them 2 % on uneven mocks.
+    const bool solo = ONE && span < most;
+    uint32_t base = 0u;
+    if (ONE) {
+        const uint32_t first = max(least_claim((uint32_t)chunk), min((uint32_t)chunk, span / (2u * gridDim.x)));
+        const uint32_t c0 = (uint32_t)min((unsigned long long)span, (unsigned long long)first * blockIdx.x);
+        base = (uint32_t)min((unsigned long long)span, (unsigned long long)first * gridDim.x);
+        if (tid == 0) {
+            q.claim = (unsigned long long)(u_lo + c0) | (unsigned long long)(u_lo + min(span, c0 + first)) << 32;
+            q.done = base >= span ? 1 : 0;
+        }
+        if (solo && lane == 0) {
+            wm.st->tab = 0;
+            wm.st->term = term_only;
+            wm.st->t_lo = u_lo;
+            wm.st->t_hi = u_hi;
+        }
+        ad.Kl = saddr(dsm) + o.hist + 4u * ((uint32_t)lane & (uint32_t)(R - 1)) + Addr<MU, R, LOGC>::shift(dp);
+    }
     __syncthreads();
 #pragma unroll 1
     for (;;) {
@@ -1474,11 +1509,18 @@ __global__ void __launch_bounds__(W * 32, 1)
         if (lane == 0) {
             const unsigned long long c = atomicAdd(&q.claim, 1ull);
             if ((uint32_t)c < (uint32_t)(c >> 32)) u = (uint32_t)c;
-            else u = claim_more(q, claim, u_lo, span, (uint32_t)chunk, status);
+            else u = claim_more<ONE>(q, claim, u_lo, base, span, (uint32_t)chunk, status);
             stay = u >= wm.st->t_lo && u < wm.st->t_hi && atomicAdd(&q.n_used[wm.st->tab], 1u) < most;
         }
         u = __shfl_sync(0xffffffffu, u, 0);
         if (!__shfl_sync(0xffffffffu, stay, 0)) {
+            if (ONE && solo) {   // no unit left
+                if (n_list) {
+                    if (V == 2) recheck_apart<MU, R, LOGC>(prm, dp, m, Tsh, wm, n_list, ad.hb(dp), lane);
+                    else recheck<MU, R, LOGC>(prm, dp, m, Tsh, wm, n_list, ad.hb(dp), lane);
+                }
+                break;
+            }
             const int k = V == 2 ? switch_table_apart<V, R, LOGC>(prm, dp, m, terms, units, ustart, Tsh, wm, q, dsm + o.hist,
                                                                   o.hstride, ad.hb(dp), u, n_list, status)
                                  : switch_table<V, R, LOGC>(prm, dp, m, terms, units, ustart, Tsh, wm, q, dsm + o.hist,
@@ -1491,6 +1533,14 @@ __global__ void __launch_bounds__(W * 32, 1)
         const Unit un = units[u];
         unit<V, R, LOGC>(prm, dp, m, Tsh, wm, ad, un, terms[un.term], lane, n_list);
     }
+    if (ONE && solo) {
+        __syncthreads();   // every warp has ended its last unit (the waits for one are bounded)
+        unsigned long long bn = drain<MU, R, LOGC, true>(prm, dp, terms, (uint32_t *)(dsm + o.hist), 0u, term_only,
+                                                         lane);
+#pragma unroll
+        for (int s2 = 16; s2 > 0; s2 >>= 1) bn += __shfl_down_sync(0xffffffffu, bn, s2);
+        if (lane == 0) wm.st->binned += bn;
+    }
     if (lane == 0) {
         atomicAdd(&stats[0], wm.st->n_cand);
         atomicAdd(&stats[1], wm.st->binned);
@@ -1499,29 +1549,30 @@ __global__ void __launch_bounds__(W * 32, 1)
     }
 }
 
-template <int V, int R, int W, int LOGC>
+template <int V, int R, int W, int LOGC, bool ONE>
 void *dkernel()
 {
-    return (void *)pairdirect_kernel<V, R, W, LOGC>;
+    return (void *)pairdirect_kernel<V, R, W, LOGC, ONE>;
 }
 
-// kernel for (mode, copies, warps, column bits); nullptr when not built
+// kernel for (mode, copies, warps, column bits), batched or for one term; nullptr when not built
+template <bool ONE>
 void *select_direct(int V, int R, int W, int logC)
 {
     if (W != DIRECT_WARPS) return nullptr;
     constexpr int DW = DIRECT_WARPS;
-    if (V == 5) return R == 1 ? dkernel<5, 1, DW, 0>() : nullptr;
-    if (V == 3) return R == 32 ? dkernel<3, 32, DW, 0>() : nullptr;
-    if (V == 4 && logC == 4) return R == 32 ? dkernel<4, 32, DW, 4>() : (R == 16 ? dkernel<4, 16, DW, 4>() : nullptr);
-    if (V == 4 && logC == 5) return R == 32 ? dkernel<4, 32, DW, 5>() : (R == 16 ? dkernel<4, 16, DW, 5>() : dkernel<4, 8, DW, 5>());
-    if (V == 4 && logC == 6) return R == 16 ? dkernel<4, 16, DW, 6>() : (R == 8 ? dkernel<4, 8, DW, 6>() : nullptr);
-    if (V == 0) return R == 32 ? dkernel<0, 32, DW, 0>() : nullptr;
-    if (V == 1 && logC == 4) return R == 32 ? dkernel<1, 32, DW, 4>() : (R == 16 ? dkernel<1, 16, DW, 4>() : nullptr);
-    if (V == 2 && logC == 4) return R == 32 ? dkernel<2, 32, DW, 4>() : (R == 16 ? dkernel<2, 16, DW, 4>() : nullptr);
-    if (V == 1 && logC == 5) return R == 32 ? dkernel<1, 32, DW, 5>() : (R == 16 ? dkernel<1, 16, DW, 5>() : dkernel<1, 8, DW, 5>());
-    if (V == 1 && logC == 6) return R == 16 ? dkernel<1, 16, DW, 6>() : (R == 8 ? dkernel<1, 8, DW, 6>() : nullptr);
-    if (V == 2 && logC == 5) return R == 32 ? dkernel<2, 32, DW, 5>() : (R == 16 ? dkernel<2, 16, DW, 5>() : dkernel<2, 8, DW, 5>());
-    if (V == 2 && logC == 6) return R == 16 ? dkernel<2, 16, DW, 6>() : (R == 8 ? dkernel<2, 8, DW, 6>() : nullptr);
+    if (V == 5) return R == 1 ? dkernel<5, 1, DW, 0, ONE>() : nullptr;
+    if (V == 3) return R == 32 ? dkernel<3, 32, DW, 0, ONE>() : nullptr;
+    if (V == 4 && logC == 4) return R == 32 ? dkernel<4, 32, DW, 4, ONE>() : (R == 16 ? dkernel<4, 16, DW, 4, ONE>() : nullptr);
+    if (V == 4 && logC == 5) return R == 32 ? dkernel<4, 32, DW, 5, ONE>() : (R == 16 ? dkernel<4, 16, DW, 5, ONE>() : dkernel<4, 8, DW, 5, ONE>());
+    if (V == 4 && logC == 6) return R == 16 ? dkernel<4, 16, DW, 6, ONE>() : (R == 8 ? dkernel<4, 8, DW, 6, ONE>() : nullptr);
+    if (V == 0) return R == 32 ? dkernel<0, 32, DW, 0, ONE>() : nullptr;
+    if (V == 1 && logC == 4) return R == 32 ? dkernel<1, 32, DW, 4, ONE>() : (R == 16 ? dkernel<1, 16, DW, 4, ONE>() : nullptr);
+    if (V == 2 && logC == 4) return R == 32 ? dkernel<2, 32, DW, 4, ONE>() : (R == 16 ? dkernel<2, 16, DW, 4, ONE>() : nullptr);
+    if (V == 1 && logC == 5) return R == 32 ? dkernel<1, 32, DW, 5, ONE>() : (R == 16 ? dkernel<1, 16, DW, 5, ONE>() : dkernel<1, 8, DW, 5, ONE>());
+    if (V == 1 && logC == 6) return R == 16 ? dkernel<1, 16, DW, 6, ONE>() : (R == 8 ? dkernel<1, 8, DW, 6, ONE>() : nullptr);
+    if (V == 2 && logC == 5) return R == 32 ? dkernel<2, 32, DW, 5, ONE>() : (R == 16 ? dkernel<2, 16, DW, 5, ONE>() : dkernel<2, 8, DW, 5, ONE>());
+    if (V == 2 && logC == 6) return R == 16 ? dkernel<2, 16, DW, 6, ONE>() : (R == 8 ? dkernel<2, 8, DW, 6, ONE>() : nullptr);
     return nullptr;
 }
 
@@ -1536,14 +1587,18 @@ size_t pairdirect_smem_bytes(const CountParams &p, int rows, int R, int C, int N
 
 cudaError_t pairdirect_set_attrs(const DirectParams &d, int mu)
 {
-    void *k = select_direct(mode_of(d, mu != 0), d.R, d.W, d.logC);
-    if (!k) return cudaErrorInvalidValue;
-    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, d.smem);
+    for (void *k : {select_direct<false>(mode_of(d, mu != 0), d.R, d.W, d.logC),
+                    select_direct<true>(mode_of(d, mu != 0), d.R, d.W, d.logC)}) {
+        if (!k) return cudaErrorInvalidValue;
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, d.smem);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 int pairdirect_max_blocks_per_sm(const DirectParams &d, int mu)
 {
-    void *k = select_direct(mode_of(d, mu != 0), d.R, d.W, d.logC);
+    void *k = select_direct<false>(mode_of(d, mu != 0), d.R, d.W, d.logC);
     int nb = 0;
     if (!k || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, d.W * 32, d.smem) != cudaSuccess) {
         cudaGetLastError();
@@ -1556,9 +1611,9 @@ cudaError_t launch_pairdirect(const CountParams &p, const DirectParams &d, const
                               const Unit *units, const uint32_t *ustart, const uint32_t *n_units, unsigned *claim,
                               unsigned long long *stats, int *status, const PairLaunch &pl, cudaStream_t s)
 {
-    void *k = select_direct(mode_of(d, p.n_mu > 1), d.R, d.W, d.logC);
+    const int term_only = pl.persistent ? -1 : pl.term, mode = mode_of(d, p.n_mu > 1);
+    void *k = pl.persistent ? select_direct<false>(mode, d.R, d.W, d.logC) : select_direct<true>(mode, d.R, d.W, d.logC);
     if (!k) return cudaErrorInvalidValue;
-    const int term_only = pl.persistent ? -1 : pl.term;
     void *args[] = {(void *)&p,       (void *)&d,     (void *)&m,     (void *)&terms,  (void *)&units,     (void *)&ustart,
                     (void *)&n_units, (void *)&claim, (void *)&stats, (void *)&status, (void *)&term_only, (void *)&pl.chunk};
     return cudaLaunchKernel(k, dim3(pl.blocks), dim3(d.W * 32), args, (size_t)d.smem, s);
