@@ -223,6 +223,7 @@ int tpcf_create(tpcf_ctx **out, int cuda_device)
     }
     if (const char *v = std::getenv("TPCF_TEST_FAIL_ALLOC")) ctx->fail_alloc_at = std::atoll(v);
     if (const char *v = std::getenv("TPCF_TEST_FAIL_COUNT")) ctx->fail_count_at = std::atoll(v);
+    if (const char *v = std::getenv("TPCF_TEST_GROUP")) ctx->test_group = std::max(1, std::atoi(v));
     if (const char *v = std::getenv("TPCF_TEST_MAX_CLUSTER")) ctx->test_max_cluster = std::atoi(v);
     *out = ctx;
     return TPCF_OK;

@@ -1001,6 +1001,7 @@ extern "C" int tpcf_count(tpcf_ctx *ctx, const tpcf_mock *mocks, int n_mock, con
     Tuned cfg;
     if (ctx->subdiv_pin) {
         cfg.subdiv = ctx->subdiv_pin;
+        cfg.group = ctx->test_group;
     } else if (ctx->autotune && mode == TPCF_PER_LAUNCH && n_mock > 0) {
         // the per-launch path runs the configuration tuned for the batched one, if any
         auto it = ctx->tune_cache.find(tune_key(ctx, mocks, n_mock, binning, terms));

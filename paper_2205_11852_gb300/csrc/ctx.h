@@ -86,11 +86,12 @@ struct tpcf_ctx {
     int test_skip_mma = 0;
     // test hooks read from the environment at tpcf_create: the n-th device
     // allocation of ensure() fails (TPCF_TEST_FAIL_ALLOC=n), the n-th
-    // tpcf_count fails as if a launch had failed (TPCF_TEST_FAIL_COUNT=n), and
-    // the device is taken to run clusters of at most n blocks (TPCF_TEST_MAX_CLUSTER=n)
+    // tpcf_count fails as if a launch had failed (TPCF_TEST_FAIL_COUNT=n), the
+    // device is taken to run clusters of at most n blocks (TPCF_TEST_MAX_CLUSTER=n),
+    // and counts of a pinned subdivision use units of n cells (TPCF_TEST_GROUP=n)
     long long fail_alloc_at = 0, n_alloc = 0;
     long long fail_count_at = 0, n_count = 0;
-    int test_max_cluster = 0;
+    int test_max_cluster = 0, test_group = 1;
     // host-input counts in groups: the groups' copies run on copy_stream;
     // pipe_ev holds [0] the call's start, [1] its end (the next call's copies
     // wait for it), then per group g [2 + 2 g] copied and [3 + 2 g] counted

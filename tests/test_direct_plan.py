@@ -86,3 +86,11 @@ def test_a_unit_never_passes_a_counter(plan, name, max_cat):
     if got:
         assert got[0] < 2 ** 32
         assert copies is None or got[1] == copies
+
+
+# the tables that the schedule tests count on: four, two and one per block, copied or with a column per |mu| bin
+@pytest.mark.parametrize("n_s,n_mu,tables,copies", [(12, 1, 4, 32), (20, 5, 2, 16), (40, 10, 2, 8), (60, 10, 1, 8),
+                                                    (30, 25, 2, 1)])
+def test_tables_per_block(plan, n_s, n_mu, tables, copies):
+    _, r, nt = plan(np.linspace(0.0, 24.0, n_s + 1), n_mu, 3000, L=100.0)
+    assert (nt, r) == (tables, copies)
