@@ -145,8 +145,8 @@ int prepare(tpcf_ctx *ctx, const tpcf_mock *mocks, int n_mock, const tpcf_binnin
     }
     // The pair counters add into 32-bit shared-memory counters: one unit adds
     // at most chunk x (points of one catalogue) pairs to any counter, which
-    // must stay below 2^32 (the direct counter drains before the sum over
-    // units could reach 2^31).
+    // must stay below 2^32 (the direct counter drains a table before the sum
+    // over units could pass 2^32 - 1, and refuses plans whose single unit could).
     if (max_cat > 0) {
         const unsigned long long cap = ((1ull << 32) - 1) / max_cat;
         if (cap < 16) return fail(ctx, TPCF_ERR_RANGE, "a catalogue above 2^28 points would overflow the 32-bit pair counters");

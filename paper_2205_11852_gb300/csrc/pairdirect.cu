@@ -63,7 +63,7 @@
 //
 // Histogram.  R copies of a (n_s + 1) x C table of 32-bit counters, lane l
 // adding to copy l mod R, so the 32 adds of a warp fall in distinct banks
-// (R = 32) or at most two per bank (R = 16).  mu is binned by sign, C =
+// (R = 32) or at most two (R = 16) or four (R = 8) per bank.  mu is binned by sign, C =
 // 2 n_mu + 2 columns from -n_mu - 1 to n_mu, and folded to |mu| when a table is
 // drained into the term's int64 histogram: when the block's last warp leaves
 // the term, or before its 32-bit counters could wrap.
@@ -103,7 +103,7 @@ struct Sched {
 constexpr int FREE = -1, DRAINING = -2;
 constexpr int FOLD_PAD = DIRECT_FOLD_PAD;   // words before a table of one copy (mode 5)
 
-// Shared memory: the block's one or two tables, T, the schedule, then one
+// Shared memory: the block's tables (one to four), T, the schedule, then one
 // region per warp: a-records (3 float4 per a-point), the b buffer (float4: x, y, z in
 // bins and the b index), the unit's runs (first index, offset in the
 // concatenation) and the recheck list.
@@ -821,10 +821,10 @@ __device__ __forceinline__ void load_tile(const float4 *buf, uint32_t nb, int la
 // the a-chunk's own cell (an auto count), of whose pairs only a < b count.
 // Padding slots hold far-away points whose adds land in the spare last row.
 // The a-points run two at a time, the last of an odd chunk alone.  The
-// pairs of one a-point or their
-// uncertainty into one predicate per lane; when any lane's is set, the
-// a-points' pairs are recomputed with a flag each, and each uncertain pair's
-// add is taken back and the pair joins the recheck list.
+// uncertainties of one a-point's pairs are or-ed into one predicate per lane;
+// when any lane's is set, the a-points' pairs are recomputed with a flag each,
+// and each uncertain pair's add is taken back and the pair joins the recheck
+// list.
 template <int V, int R, int LOGC, bool CHK>
 __device__ __forceinline__ void tile(const CountParams &prm, const DirectParams &dp, const Mesh &m,
                                      const unsigned long long *T, const WarpMem &wm,

@@ -407,9 +407,7 @@ bool build_direct(const tpcf_binning &b, const Plan &pl, int smem_sm, int smem_b
     double unit = b.s_edges[geo ? 0 : 1], la = 0.0, dev = 0.0;
     // Linear edges whose width is not a short binary fraction (150 / 23) are
     // k widths but for a rounding each: dev is how far, in bins, and widens the
-    // band of pairs that are rechecked against the exact thresholds.  They are
-    // the rule: 90 of the 116 binnings of 12 to 40 bins up to 120, 150, 160 or
-    // 200 Mpc/h.
+    // band of pairs that are rechecked against the exact thresholds.
     if (!geo && !p.linear) {
         unit = b.s_edges[b.n_s] / b.n_s;
         for (int k = 1; k <= b.n_s; k++) dev = std::max(dev, std::fabs(b.s_edges[k] / unit - k));
