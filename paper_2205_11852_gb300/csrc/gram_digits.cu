@@ -105,7 +105,7 @@ __device__ __forceinline__ long long to_fixed(double y, int e)
 // element (the sum and the residual) bound the two kernels.
 __global__ void __launch_bounds__(32 * COL_WARPS)
     digits_kernel(const double *__restrict__ x0, const double *__restrict__ x1, const double *__restrict__ x2,
-                  const ColPartial *__restrict__ part, int n_mock, int nbin, int n_rb, int n_ks,
+                  const ColRange *__restrict__ part, int n_mock, int nbin, int n_rb, int n_ks,
                   unsigned char *__restrict__ tiles, int *__restrict__ ecol, double *__restrict__ mean,
                   uint32_t *__restrict__ oct)
 {
@@ -113,11 +113,11 @@ __global__ void __launch_bounds__(32 * COL_WARPS)
     const int v = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const double *x = v == 0 ? x0 : (v == 1 ? x1 : x2);
     const int b = blockIdx.x * 32 + lane;
-    double mu, mn, mx;
+    double mu;
     for (int k = threadIdx.x; k < OCT * 32; k += blockDim.x) cnt[k / 32][k % 32] = 0u;
-    column_stats(part, v, n_mock, nbin, b, mu, mn, mx);   // (has block barriers)
+    const ColRange range = column_stats(part, v, n_mock, nbin, b, mu);   // (has block barriers)
     // |x - mean| is largest at an extremum (rounding is monotone); NaN and infinities fail the tests
-    const double top = fmax(mx - mu, mu - mn);
+    const double top = fmax(of_key(range.hi) - mu, mu - of_key(range.lo));
     const bool bad = !(mu == mu) || !(top < 0x1p400) || (top != 0.0 && !(top > 0x1p-400));
     const int e = bad || top == 0.0 ? 0 : ilogb(top) + 1;
     if (blockIdx.y == 0 && warp == 0 && b < nbin) {
@@ -510,7 +510,7 @@ DShape dshape(int n_mock, int nbin, int n_var, int n_sm)
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     s.o_T = al((size_t)n_var * s.n_rb * s.n_ks * SLICE_BYTES);
     s.o_part = s.o_T + al((size_t)s.n_seg * n_var * nbin * nbin * sizeof(longlong2));
-    s.o_mean = s.o_part + al((size_t)n_var * COL_CHUNKS * nbin * sizeof(ColPartial));
+    s.o_mean = s.o_part + al((size_t)n_var * COL_CHUNKS * nbin * sizeof(ColRange));
     s.o_e = s.o_mean + al((size_t)n_var * nbin * 8);
     s.o_oct = s.o_e + al((size_t)n_var * nbin * 4);
     s.bytes = s.o_oct + al((size_t)n_var * OCT * nbin * 4);
@@ -544,9 +544,9 @@ cudaError_t launch_cov_digits(const double *x0, const double *x1, const double *
     longlong2 *T = (longlong2 *)(w + d.o_T);
     double *mean = (double *)(w + d.o_mean);
     int *ecol = (int *)(w + d.o_e);
-    ColPartial *part = (ColPartial *)(w + d.o_part);
+    ColRange *part = (ColRange *)(w + d.o_part);
     uint32_t *oct = (uint32_t *)(w + d.o_oct);
-    cudaError_t e = launch_column_partials(x0, x1, x2, n_var, n_mock, nbin, part, s, oct, OCT);
+    cudaError_t e = launch_column_partials(x0, x1, x2, n_var, n_mock, nbin, part, oct, OCT, s);
     if (e != cudaSuccess) return e;
     digits_kernel<<<dim3((nbin + 31) / 32, COL_CHUNKS, n_var), 32 * COL_WARPS, 0, s>>>(x0, x1, x2, part, n_mock, nbin,
                                                                                       d.n_rb, d.n_ks, w, ecol, mean, oct);

@@ -166,7 +166,7 @@ __device__ __forceinline__ void split_bf16(double d, uint16_t (&p)[3])
 template <int PREC>
 __global__ void __launch_bounds__(32 * COL_WARPS)
     split_kernel(const double *__restrict__ x0, const double *__restrict__ x1, const double *__restrict__ x2,
-                 const ColPartial *__restrict__ part, int n_mock, int nbin, int n_rb, int n_ks,
+                 const ColSum *__restrict__ part, int n_mock, int nbin, int n_rb, int n_ks,
                  unsigned char *__restrict__ tiles)
 {
     constexpr int TB = tile_bytes<PREC>();
@@ -175,8 +175,8 @@ __global__ void __launch_bounds__(32 * COL_WARPS)
     const int v = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const double *x = v == 0 ? x0 : (v == 1 ? x1 : x2);
     const int b = blockIdx.x * 32 + lane;
-    double mu, mn, mx;
-    column_stats(part, v, n_mock, nbin, b, mu, mn, mx);
+    double mu;
+    column_stats(part, v, n_mock, nbin, b, mu);
     if (b >= nbin) return;
     const int rb = b / TM, r = b % TM;
     const int n_g = n_ks * (KS / per), share = (n_g + (int)gridDim.y - 1) / (int)gridDim.y;
@@ -560,7 +560,7 @@ size_t work_bytes_of(int n_mock, int nbin, int n_var, int n_sm)
     const Chunking c = chunking(n_mock, nbin, n_var, n_sm);
     const size_t g = (size_t)n_var * nbin * nbin * 8;
     return al256(tiles_bytes<PREC>(n_mock, nbin, n_var)) + al256((size_t)c.n_kc * g) +
-           al256((size_t)n_var * COL_CHUNKS * nbin * sizeof(ColPartial));
+           al256((size_t)n_var * COL_CHUNKS * nbin * sizeof(ColSum));
 }
 
 // n_var = 3: the LC covariance of (x0, x1, x2); n_var = 1: the sample covariance of x0 into C_lc
@@ -579,10 +579,10 @@ cudaError_t run(const double *x0, const double *x1, const double *x2, int n_var,
     size_t o = al256(tiles_bytes<PREC>(n_mock, nbin, n_var));
     double *P = (double *)(w + o);
     o += al256((size_t)ch.n_kc * g * 8);
-    ColPartial *part = (ColPartial *)(w + o);
-    o += al256((size_t)n_var * COL_CHUNKS * nbin * sizeof(ColPartial));
+    ColSum *part = (ColSum *)(w + o);
+    o += al256((size_t)n_var * COL_CHUNKS * nbin * sizeof(ColSum));
     if (o > work_bytes) return cudaErrorInvalidValue;
-    cudaError_t e = launch_column_partials(x0, x1, x2, n_var, n_mock, nbin, part, s);
+    cudaError_t e = launch_column_partials(x0, x1, x2, n_var, n_mock, nbin, part, nullptr, 0, s);
     if (e != cudaSuccess) return e;
     split_kernel<PREC><<<dim3((nbin + 31) / 32, COL_CHUNKS, n_var), 32 * COL_WARPS, 0, s>>>(x0, x1, x2, part, n_mock,
                                                                                            nbin, n_rb, n_ks, tiles);

@@ -1389,8 +1389,9 @@ __device__ __forceinline__ int switch_table(const CountParams &prm, const Direct
     if (u != NO_UNIT && lane == 0) {
         const int t = units[u].term;
         const uint32_t t_lo = ustart[(size_t)t * dp.n_groups], t_hi = ustart[(size_t)(t + 1) * dp.n_groups];
-        // (inlined it costs linear bins 0.6 to 1.5 %, as a call geometric ones 3 %)
-        k = is_geo(V) ? enter_table(q, dp, t) : enter_table_apart(q, dp, t);
+        // (inlined it costs linear bins with mu 0.6 to 1.5 %; as a call, geometric bins 3 % and s only, on 16 mocks of
+        // 4000 points, 1.5 %)
+        k = is_geo(V) || V == 0 ? enter_table(q, dp, t) : enter_table_apart(q, dp, t);
         if (k < 0) atomicOr(status, STATUS_TIMEOUT);
         wm.st->tab = k;
         wm.st->term = t;
