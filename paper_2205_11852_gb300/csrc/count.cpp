@@ -409,7 +409,7 @@ int enqueue(tpcf_ctx *ctx, const Setup &S, int mode, cudaStream_t s, void *small
             L.term = t;
             if (S.direct) {
                 // one launch per term over that term's units, each with its own claim counter; a block's
-                // first claim is its by number, further ones shrink (see pairdirect_kernel)
+                // first claim follows from its number, further ones shrink (see pairdirect_kernel)
                 L.blocks = S.blocks;
                 L.chunk = std::max(1, S.claim_units);
                 CK(launch_pairdirect(prm, S.dp, mesh, d_terms, (const Unit *)S.units, ust, ust + (S.ntc - 1),

@@ -1476,14 +1476,14 @@ __global__ void __launch_bounds__(W * 32, 1)
     const uint32_t span = u_hi - u_lo;
     const unsigned most = most_units(dp);
     Addr<MU, R, LOGC> ad{0u};
-    // One launch per term: a block's first claim is its by number (of the size
-    // the counter would give), and its warps start in the term's table and leave
-    // it together, unless the term is long enough to fill it.  Small terms'
+    // One launch per term: a block's first claim follows from its number (its
+    // size is what the counter would give), and its warps start in the term's
+    // table and leave it together, unless the term is long enough to fill it.  Small terms'
     // launches are too short for 16 warps to pass the lock and the counter one
     // after another: 16 mocks of 4000 points, whole step, 3.33 -> 2.34 ms; one
     // mock and 50 subsets of 50 000 points 28.9 -> 27.1.  Kernels of their own,
-    // since the branches cost batched launches 1 %; first claims by number cost
-    // them 2 % on uneven mocks.
+    // since the branches cost batched launches 1 %; first claims by block number
+    // cost them 2 % on uneven mocks.
     const bool solo = ONE && span < most;
     uint32_t base = 0u;
     if (ONE) {
